@@ -330,145 +330,149 @@ void launch_pose_batched(const void* args, const BlockMap* map, int nblocks, cud
 // ------------------------------------------------------------------------------------------
 struct CellBound { float fmax, fmin; };
 
-// Displacement x - c: with mi, the minimum image on periodic axes; without, the plain difference
-// (control points staged at the brick's nearest image, valid for every point of the brick).
+// Bounds of Eq. 3 over a ball of radius h about (x, y, z) from the wrapped control points: every
+// one is at least r - h and at most r + h away. Fast reciprocal/sqrt: the 1e-3 decision margins
+// dwarf their error. (Bricks whose candidates do not fit the staging; the others take pair_bound.)
+__device__ __forceinline__ CellBound bound_at(const float4* cw, int c0, int c1, float x, float y, float z, float h,
+                                              const Geom& g) {
+  CellBound b{0.0f, 0.0f};
+  for (int i = c0; i < c1; ++i) {
+    const float4 c = cw[i];
+    const float dx = min_image_rn(x - c.x, (float)g.n[0], g.wall[0]);
+    const float dy = min_image_rn(y - c.y, (float)g.n[1], g.wall[1]);
+    const float dz = min_image_rn(z - c.z, (float)g.n[2], g.wall[2]);
+    const float r2 = dx * dx + dy * dy + dz * dz;
+    const float r = r2 * rsqrtf(fmaxf(r2, 1e-30f));
+    const float rmin = fmaxf(r - h, 1e-15f), rmax = r + h;
+    b.fmax += __fdividef(c.w, rmin * rmin);
+    b.fmin += __fdividef(c.w, rmax * rmax);
+  }
+  return b;
+}
+
+// Whole-cell mask evaluated by one thread from the wrapped control points (same bricks): the fast
+// value, and within 4e-5 of 1 the exact binary32 sequence. Bit s = a + 4 b + 16 c is sub-sample
+// (a, b, c) of cell (i, j, k).
+__device__ uint64_t particle_mask_serial(const float4* cw, int c0, int c1, int i, int j, int k, const Geom& g) {
+  uint64_t m = 0ull;
+  for (int s = 0; s < 64; ++s) {
+    const float x = (float)i + (0.125f + 0.25f * (float)(s & 3)), y = (float)j + (0.125f + 0.25f * (float)((s >> 2) & 3)),
+                z = (float)k + (0.125f + 0.25f * (float)(s >> 4));
+    const float f = metaball_value(cw, c0, c1, x, y, z, g);
+    const bool in = fabsf(f - 1.0f) > 4e-5f ? f >= 1.0f : metaball_exact(cw, c0, c1, x, y, z, g) >= 1.0f;
+    if (in) m |= 1ull << s;
+  }
+  return m;
+}
+
+__device__ __forceinline__ float fast_rcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Two control points as the staging holds them: {x0, x1, y0, y1}, {z0, z1, k0, k1}. A particle with
+// an odd number of points ends with a far point of weight 0.
+struct CenterPair { float4 xy, zk; };
+__device__ __forceinline__ CenterPair load_pair(const float4* cw, int q) { return CenterPair{cw[2 * q], cw[2 * q + 1]}; }
+// Displacement x - c: with MI the minimum image on a periodic axis; without, the plain difference
+// (points staged at the brick's nearest image, valid for every point of the brick).
 template <bool MI>
 __device__ __forceinline__ float disp(float x, float c, int a, const Geom& g) {
   return MI ? min_image_rn(x - c, (float)g.n[a], g.wall[a]) : x - c;
 }
-
-// Bounds of Eq. 3 over a ball of radius h about (x, y, z): every control point is at least
-// r - h and at most r + h away. Fast reciprocal/sqrt: the 1e-3 decision margins dwarf their error.
-template <bool MI>
-__device__ __forceinline__ CellBound bound_at_t(const float4* cw, int c0, int c1, float x, float y, float z,
-                                                float h, const Geom& g) {
-  float fmax = 0.0f, fmin = 0.0f;
-  for (int i = c0; i < c1; ++i) {
-    const float4 c = cw[i];
-    const float dx = disp<MI>(x, c.x, 0, g), dy = disp<MI>(y, c.y, 1, g), dz = disp<MI>(z, c.z, 2, g);
-    const float r2 = dx * dx + dy * dy + dz * dz;
-    const float r = r2 * rsqrtf(fmaxf(r2, 1e-30f));
-    const float rmin = fmaxf(r - h, 1e-15f), rmax = r + h;
-    fmax += __fdividef(c.w, rmin * rmin);
-    fmin += __fdividef(c.w, rmax * rmax);
-  }
-  CellBound b;
-  b.fmax = fmax;
-  b.fmin = fmin;
-  return b;
+// acc + k0 / r0 + k1 / r1 with one reciprocal (the reciprocal unit is a quarter as wide as the
+// multiply-add pipe): r0 = 0 gives infinity, r0 = r1 = 0 NaN, which callers send to the exact test.
+__device__ __forceinline__ float add_quotients(float acc, float k0, float r0, float k1, float r1) {
+  return fmaf(fmaf(k0, r1, k1 * r0), fast_rcp(r0 * r1), acc);
 }
 
-// Upper/lower bounds over a ball of radius h1 and the upper bound over radius h2 (one pass).
+// Bounds of Eq. 3 over the ball of radius h1 about (x, y, z), and with TWO its upper bound over radius
+// h2 as well, from the staged pairs q0 .. q1 - 1.
 struct Bound2 { float fmax1, fmin1, fmax2; };
-template <bool MI>
-__device__ __forceinline__ Bound2 bound_two_t(const float4* cw, int c0, int c1, float x, float y, float z,
-                                              float h1, float h2, const Geom& g) {
+template <bool MI, bool TWO>
+__device__ __forceinline__ Bound2 pair_bound(const float4* cw, int q0, int q1, float x, float y, float z, float h1,
+                                             float h2, const Geom& g) {
   Bound2 b{0.0f, 0.0f, 0.0f};
-  for (int i = c0; i < c1; ++i) {
-    const float4 c = cw[i];
-    const float dx = disp<MI>(x, c.x, 0, g), dy = disp<MI>(y, c.y, 1, g), dz = disp<MI>(z, c.z, 2, g);
-    const float r2 = dx * dx + dy * dy + dz * dz;
-    const float r = r2 * rsqrtf(fmaxf(r2, 1e-30f));
-    const float a = fmaxf(r - h1, 1e-15f), bb = r + h1, cc = fmaxf(r - h2, 1e-15f);
-    b.fmax1 += __fdividef(c.w, a * a);
-    b.fmin1 += __fdividef(c.w, bb * bb);
-    b.fmax2 += __fdividef(c.w, cc * cc);
+  for (int q = q0; q < q1; ++q) {
+    const CenterPair c = load_pair(cw, q);
+    const float dx0 = disp<MI>(x, c.xy.x, 0, g), dx1 = disp<MI>(x, c.xy.y, 0, g), dy0 = disp<MI>(y, c.xy.z, 1, g),
+                dy1 = disp<MI>(y, c.xy.w, 1, g), dz0 = disp<MI>(z, c.zk.x, 2, g), dz1 = disp<MI>(z, c.zk.y, 2, g);
+    const float s0 = dx0 * dx0 + dy0 * dy0 + dz0 * dz0, s1 = dx1 * dx1 + dy1 * dy1 + dz1 * dz1;
+    const float r0 = s0 * rsqrtf(fmaxf(s0, 1e-30f)), r1 = s1 * rsqrtf(fmaxf(s1, 1e-30f));
+    const float a0 = fmaxf(r0 - h1, 1e-9f), a1 = fmaxf(r1 - h1, 1e-9f), b0 = r0 + h1, b1 = r1 + h1;
+    b.fmax1 = add_quotients(b.fmax1, c.zk.z, a0 * a0, c.zk.w, a1 * a1);
+    b.fmin1 = add_quotients(b.fmin1, c.zk.z, b0 * b0, c.zk.w, b1 * b1);
+    if (TWO) {
+      const float d0 = fmaxf(r0 - h2, 1e-9f), d1 = fmaxf(r1 - h2, 1e-9f);
+      b.fmax2 = add_quotients(b.fmax2, c.zk.z, d0 * d0, c.zk.w, d1 * d1);
+    }
   }
   return b;
 }
 
-// Sub-sample inside test: fast value from the staged control points; within 4e-5 of 1 the
-// exact binary32 sequence shared with the CPU oracle decides, on the original wrapped points.
+// The sub-samples (x, y, z) and (x, y, z + 1/2) of one lane in one pass over the staged pairs: fast
+// values (error ~1e-6 relative); within 4e-5 of 1, or not a number, the exact binary32 sequence
+// shared with the CPU oracle decides, on the original wrapped points e0 .. e1 - 1.
 template <bool MI>
-__device__ __forceinline__ bool subsample_inside_t(const float4* cw, int c0, int c1, const float4* cw_exact,
-                                                   int e0, int e1, float x, float y, float z, const Geom& g) {
-  float f = 0.0f;
-  for (int i = c0; i < c1; ++i) {
-    const float4 c = cw[i];
-    const float dx = disp<MI>(x, c.x, 0, g), dy = disp<MI>(y, c.y, 1, g), dz = disp<MI>(z, c.z, 2, g);
-    f += __fdividef(c.w, dx * dx + dy * dy + dz * dz);
-  }
-  if (fabsf(f - 1.0f) > 4e-5f) return f >= 1.0f;
-  return metaball_exact(cw_exact, e0, e1, x, y, z, g) >= 1.0f;
-}
-
-// Two sub-samples of one lane that differ only in z (z and z + 1/2), in one pass over the
-// staged control points: the point load, the x/y displacements and dx^2 + dy^2 are shared.
-// Same fast-value tolerance and exact fallback as subsample_inside_t.
-template <bool MI>
-__device__ __forceinline__ void subsample_pair_t(const float4* cw, int c0, int c1, const float4* cw_exact, int e0,
-                                                 int e1, float x, float y, float z, const Geom& g, bool& in_lo,
-                                                 bool& in_hi) {
+__device__ __forceinline__ void subsample_pair(const float4* cw, int q0, int q1, const float4* cw_exact, int e0, int e1,
+                                               float x, float y, float z, const Geom& g, bool& in_lo, bool& in_hi) {
   const float zh = z + 0.5f;
   float flo = 0.0f, fhi = 0.0f;
-  for (int i = c0; i < c1; ++i) {
-    const float4 c = cw[i];
-    const float dx = disp<MI>(x, c.x, 0, g), dy = disp<MI>(y, c.y, 1, g);
-    const float dzl = disp<MI>(z, c.z, 2, g), dzh = disp<MI>(zh, c.z, 2, g);
-    const float rxy = dx * dx + dy * dy;
-    flo += __fdividef(c.w, rxy + dzl * dzl);
-    fhi += __fdividef(c.w, rxy + dzh * dzh);
+  for (int q = q0; q < q1; ++q) {
+    const CenterPair c = load_pair(cw, q);
+    const float dx0 = disp<MI>(x, c.xy.x, 0, g), dx1 = disp<MI>(x, c.xy.y, 0, g), dy0 = disp<MI>(y, c.xy.z, 1, g),
+                dy1 = disp<MI>(y, c.xy.w, 1, g);
+    const float l0 = disp<MI>(z, c.zk.x, 2, g), l1 = disp<MI>(z, c.zk.y, 2, g), h0 = disp<MI>(zh, c.zk.x, 2, g),
+                h1 = disp<MI>(zh, c.zk.y, 2, g);
+    const float r0 = dx0 * dx0 + dy0 * dy0, r1 = dx1 * dx1 + dy1 * dy1;
+    flo = add_quotients(flo, c.zk.z, r0 + l0 * l0, c.zk.w, r1 + l1 * l1);
+    fhi = add_quotients(fhi, c.zk.z, r0 + h0 * h0, c.zk.w, r1 + h1 * h1);
   }
   in_lo = fabsf(flo - 1.0f) > 4e-5f ? flo >= 1.0f : metaball_exact(cw_exact, e0, e1, x, y, z, g) >= 1.0f;
   in_hi = fabsf(fhi - 1.0f) > 4e-5f ? fhi >= 1.0f : metaball_exact(cw_exact, e0, e1, x, y, zh, g) >= 1.0f;
 }
 
-// Runtime dispatch on the (warp-uniform) minimum-image switch.
-__device__ __forceinline__ CellBound bound_at(const float4* cw, int c0, int c1, float x, float y, float z,
-                                              float h, const Geom& g, bool mi = true) {
-  return mi ? bound_at_t<true>(cw, c0, c1, x, y, z, h, g) : bound_at_t<false>(cw, c0, c1, x, y, z, h, g);
-}
-__device__ __forceinline__ Bound2 bound_two(const float4* cw, int c0, int c1, float x, float y, float z,
-                                            float h1, float h2, const Geom& g, bool mi) {
-  return mi ? bound_two_t<true>(cw, c0, c1, x, y, z, h1, h2, g) : bound_two_t<false>(cw, c0, c1, x, y, z, h1, h2, g);
-}
-__device__ __forceinline__ bool subsample_inside(const float4* cw, int c0, int c1, bool mi,
-                                                 const float4* cw_exact, int e0, int e1, float x, float y,
-                                                 float z, const Geom& g) {
-  return mi ? subsample_inside_t<true>(cw, c0, c1, cw_exact, e0, e1, x, y, z, g)
-            : subsample_inside_t<false>(cw, c0, c1, cw_exact, e0, e1, x, y, z, g);
-}
-
-// Sub-sample s (bit s = a + 4 b + 16 c) of cell (i, j, k) inside the particle?
-__device__ __forceinline__ bool subsample_bit(const float4* cw, int c0, int c1, bool mi, const float4* cw_exact,
-                                              int e0, int e1, int i, int j, int k, int s, const Geom& g) {
-  const int a = s & 3, b = (s >> 2) & 3, cc = s >> 4;
-  return subsample_inside(cw, c0, c1, mi, cw_exact, e0, e1, (float)i + (0.125f + 0.25f * (float)a),
-                          (float)j + (0.125f + 0.25f * (float)b), (float)k + (0.125f + 0.25f * (float)cc), g);
-}
-
-// Whole-cell mask evaluated by one thread (fallback when the shared queue is full).
-__device__ uint64_t particle_mask_serial(const float4* cw, int c0, int c1, bool mi, const float4* cw_exact, int e0,
-                                         int e1, int i, int j, int k, const Geom& g) {
-  uint64_t m = 0ull;
-  for (int s = 0; s < 64; ++s)
-    if (subsample_bit(cw, c0, c1, mi, cw_exact, e0, e1, i, j, k, s, g)) m |= 1ull << s;
-  return m;
-}
-
-constexpr int RW_WARPS = 8;        // warps (bricks in flight) per block
-constexpr int RW_CENTERS = 192;    // control points one warp stages
+constexpr int RW_WARPS = 8;        // warps (pieces in flight) per block
+constexpr int RW_CENTERS = 192;    // control points one warp stages (even)
 constexpr int RW_CAND = 8;         // candidates one warp stages (more: the unstaged path)
+constexpr int RW_LISTED = 0xffff;  // marks a mini-brick whose cells are evaluated one by one
 
 struct RasterWarp {
-  float4 cw[RW_CENTERS];           // control points at the brick's nearest image
-  unsigned char mcls[RW_CAND][64]; // per candidate and mini-brick: class | walker bit << 2
-  int p[RW_CAND], c0[RW_CAND], c1[RW_CAND], e0[RW_CAND], cls[RW_CAND];
+  float4 cw[RW_CENTERS];            // control point pairs at the brick's nearest image
+  unsigned char mcls[RW_CAND][64];  // per candidate and mini-brick: class | walker bit << 2
+  uint16_t val[64];                 // per mini-brick: the solid word of all its cells, or RW_LISTED
+  unsigned char list[64];           // the mini-bricks whose cells are evaluated
+  int p[RW_CAND], q0[RW_CAND], q1[RW_CAND], e0[RW_CAND], e1[RW_CAND];
 };
 
-// One warp per brick of the raster list (grid-stride over warps; no block barriers):
+// Pieces a brick is cut into, as a power of two: a brick's straddling cells are one warp's serial
+// work (up to ~100 evaluations of 64 sub-samples, ~1 us each), so a list shorter than four per
+// resident warp is spread over them: slices of 32, 16 or 8 mini-bricks, then parts that share out a
+// slice's straddling mini-bricks down to one each. Every piece stages the candidates again, so
+// longer lists keep whole bricks (256^3, 13175 bricks on 2432 warps: 190 us whole, 267 us in
+// eighths; 96^3, 902 bricks: 97 us whole, 43 us in eighths).
+__device__ __forceinline__ int raster_pieces_log2(uint32_t nlist, uint32_t warps) {
+  int s = 0;
+  while (s < 6 && (nlist << (s + 1)) <= 4u * warps) ++s;
+  return s;
+}
+
+// One warp per piece of a brick of the raster list (pieces beyond one per warp from a work counter;
+// no block barriers):
 //  1. the brick's candidates and their control points (staged at the brick's nearest image) are
-//     gathered by the lanes in parallel, and each candidate is classified for the whole brick;
-//  2. mini-bricks (2^3 cells): raster class per candidate and the walkers' mask bit (Eq. 3 may
-//     reach 1 within sqrt(3) + the walker step margin);
-//  3. 16 rounds of 32 cells: each lane bounds Eq. 3 over its cell (outside / inside / straddling);
-//     the warp then evaluates every straddling (cell, candidate) pair together, 32 sub-samples per
-//     ballot, and the cell's lane folds the 64-bit mask in: count = popcount(OR of masks), owner =
+//     gathered by the lanes in parallel;
+//  2. the slice's mini-bricks (2^3 cells): raster class per candidate (outside / inside /
+//     straddling) and the walkers' mask bit (Eq. 3 may reach 1 within sqrt(3) + the walker step
+//     margin). Cells of mini-bricks that no candidate straddles are filled at once;
+//  3. the straddling mini-bricks, four (32 cells) per round: each lane bounds Eq. 3 over its cell; the
+//     warp then evaluates every straddling (cell, candidate) pair together, two sub-samples per
+//     lane, and the cell's lane folds the 64-bit mask in: count = popcount(OR of masks), owner =
 //     the candidate with most sub-samples, lowest index on ties.
 // All decisions use bounds with a 1e-3 margin and, within 4e-5 of f = 1, the exact binary32
 // sequence shared with the CPU oracle, so counts and owners equal the oracle's bit for bit.
-// With cells = 0 a launch stops after step 2: the IBB coupling reads node classes, not counts,
-// and needs only the walkers' masks each step.
+// With cells = 0 a launch stops after the masks of step 2: the IBB coupling reads node classes, not
+// counts, and needs only the walkers' masks each step.
 struct RasterArgs {
   Geom g;
   ParticleSet ps;
@@ -478,7 +482,7 @@ struct RasterArgs {
   int cells;
 };
 
-__device__ __forceinline__ void raster_body(const RasterArgs& A) {
+__device__ __forceinline__ void raster_body(const RasterArgs& A, int blk, int nblk) {
   const Geom g = A.g;
   const ParticleSet ps = A.ps;
   const BrickSet bs = A.bs;
@@ -490,19 +494,27 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A) {
   RasterWarp& W = s_rw[wib];
   const uint32_t nbrick = (uint32_t)g.nb[0] * g.nb[1] * g.nb[2];
   const uint32_t nlist = bs.bword[nbrick];
+  const uint32_t warps = (uint32_t)nblk * RW_WARPS;
+  // the masks alone are two rounds of bounds per brick: whole bricks there
+  const int plog = A.cells ? raster_pieces_log2(nlist, warps) : 0, slog = min(plog, 3), parts = 1 << (plog - slog);
+  const uint32_t units = nlist << plog;
+  const int K = 64 >> slog;          // mini-bricks per slice: 64, 32, 16 or 8
+  const int rows_y = K >= 16 ? 8 : 4;   // cell rows of a slice along y
   unsigned long long queued = 0;
-  // bricks are taken from a shared counter (bword[nbrick + 1], zero after the brick pass), one
-  // per warp at a time: their cost ranges from a few bound tests to ~100 straddling cells, and a
-  // fixed assignment left a long tail
-  uint32_t li = 0;
-  if (lane == 0) li = atomicAdd(&bs.bword[nbrick + 1], 1u);
-  li = __shfl_sync(full, li, 0);
-  for (; li < nlist; ) {
-    const uint32_t b = (uint32_t)bs.rlist[li];
+  // this lane's sub-samples: offsets within the cell (z and z + 1/2)
+  const float ax = 0.125f + 0.25f * (float)(lane & 3), ay = 0.125f + 0.25f * (float)((lane >> 2) & 3),
+              az = 0.125f + 0.25f * (float)(lane >> 4);
+  // the first piece by warp index, further ones from a shared counter (bword[nbrick + 1], zero
+  // after the brick pass): their cost ranges from a few bound tests to ~100 straddling cells, and
+  // a fixed assignment left a long tail
+  for (uint32_t u = (uint32_t)blk * RW_WARPS + wib; u < units;) {
+    const int slice = (int)(u & ((1u << slog) - 1u)), part = (int)(u >> slog) & (parts - 1);
+    const uint32_t b = (uint32_t)bs.rlist[u >> plog];
+    const int mb0 = slice * K;
     const int bi = b % g.nb[0], bj = (b / g.nb[0]) % g.nb[1], bk = b / (g.nb[0] * g.nb[1]);
     const uint32_t nc = bs.bword[b] & 0xffffu;
     const bool over = nc > MAXC;
-    // 1. candidates, in parallel over lanes; offsets of their control points by a warp scan
+    // 1. candidates, in parallel over lanes; offsets of their control point pairs by a warp scan
     int p = -1, cnt = 0, g0 = 0;
     if (!over && lane < (int)nc) {
       const uint16_t cid = bs.bcand[b * MAXC + lane];
@@ -514,101 +526,148 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A) {
     }
     const unsigned rel = __ballot_sync(full, p >= 0);
     const int n = __popc(rel);
-    int incl = cnt;
+    const int npair = (cnt + 1) >> 1;
+    int incl = npair;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int v = __shfl_up_sync(full, incl, o);
       if (lane >= o) incl += v;
     }
     const int tot = __shfl_sync(full, incl, 31);
-    const bool staged = !over && n <= RW_CAND && tot <= RW_CENTERS;
+    const bool staged = !over && n <= RW_CAND && 2 * tot <= RW_CENTERS;
     if (staged && p >= 0) {
       const int slot = __popc(rel & ((1u << lane) - 1u));
-      W.p[slot] = p; W.c0[slot] = incl - cnt; W.c1[slot] = incl; W.e0[slot] = g0;
+      W.p[slot] = p; W.q0[slot] = incl - npair; W.q1[slot] = incl; W.e0[slot] = g0; W.e1[slot] = g0 + cnt;
     }
     __syncwarp();
     bool mi = true;
+    int nlisted = 0;
     if (staged) {
       const float bc[3] = {(float)(bi * BRICK) + 4.0f, (float)(bj * BRICK) + 4.0f, (float)(bk * BRICK) + 4.0f};
       const float H = 6.0f + ps.walk_margin;
       bool near_half = false;
       for (int m = 0; m < n; ++m) {
-        const int len = W.c1[m] - W.c0[m];
-        for (int i = lane; i < len; i += 32) {
-          float4 cc = bs.cworld[W.e0[m] + i];
-          float* v[3] = {&cc.x, &cc.y, &cc.z};
+        const int len = W.e1[m] - W.e0[m], slots = 2 * (W.q1[m] - W.q0[m]);
+        for (int i = lane; i < slots; i += 32) {
+          float v[3] = {bc[0] + 1e4f, bc[1], bc[2]}, k = 0.0f;   // the far point of an odd count
+          if (i < len) {
+            const float4 cc = bs.cworld[W.e0[m] + i];
+            v[0] = cc.x; v[1] = cc.y; v[2] = cc.z; k = cc.w;
 #pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            if (g.wall[a]) continue;
-            const float na = (float)g.n[a];
-            const float d = *v[a] - bc[a];
-            if (d > 0.5f * na) *v[a] -= na; else if (d < -0.5f * na) *v[a] += na;
-            if (fabsf(*v[a] - bc[a]) > 0.5f * na - H) near_half = true;
+            for (int a = 0; a < 3; ++a) {
+              if (g.wall[a]) continue;
+              const float na = (float)g.n[a];
+              const float d = v[a] - bc[a];
+              if (d > 0.5f * na) v[a] -= na; else if (d < -0.5f * na) v[a] += na;
+              if (fabsf(v[a] - bc[a]) > 0.5f * na - H) near_half = true;
+            }
           }
-          W.cw[W.c0[m] + i] = cc;
+          float* w = reinterpret_cast<float*>(W.cw + 2 * (W.q0[m] + (i >> 1))) + (i & 1);
+          w[0] = v[0]; w[2] = v[1]; w[4] = v[2]; w[6] = k;
         }
       }
       mi = __any_sync(full, near_half);
       __syncwarp();
-      if (lane < n) {   // brick-level class (sub-samples lie within the half-diagonal of the brick)
-        const float ex0 = (float)(bi * BRICK), ex1 = fminf((float)((bi + 1) * BRICK), (float)g.n[0]);
-        const float ey0 = (float)(bj * BRICK), ey1 = fminf((float)((bj + 1) * BRICK), (float)g.n[1]);
-        const float ez0 = (float)(bk * BRICK), ez1 = fminf((float)((bk + 1) * BRICK), (float)g.n[2]);
-        const float hx = 0.5f * (ex1 - ex0) - 0.125f, hy = 0.5f * (ey1 - ey0) - 0.125f, hz = 0.5f * (ez1 - ez0) - 0.125f;
-        const CellBound bb = bound_at(W.cw, W.c0[lane], W.c1[lane], 0.5f * (ex0 + ex1), 0.5f * (ey0 + ey1),
-                                      0.5f * (ez0 + ez1), sqrtf(hx * hx + hy * hy + hz * hz), g, mi);
-        W.cls[lane] = bb.fmax < 0.999f ? 0 : (bb.fmin > 1.001f ? 1 : 2);
-      }
-      __syncwarp();
       // 2. mini-bricks: raster class and walker bit per candidate
-      for (int pr = lane; pr < 64 * n; pr += 32) {
-        const int mb = pr & 63, m = pr >> 6;
+      const float hw = 1.7320508f + ps.walk_margin;
+      for (int pr = lane; pr < K * n; pr += 32) {
+        const int mb = mb0 + (pr & (K - 1)), m = pr >> (6 - slog);
         const float xm = (float)(bi * BRICK + 2 * (mb & 3)) + 1.0f, ym = (float)(bj * BRICK + 2 * ((mb >> 2) & 3)) + 1.0f,
                     zm = (float)(bk * BRICK + 2 * (mb >> 4)) + 1.0f;
-        int cls = W.cls[m];
-        bool need;
-        if (cls == 2) {
-          const Bound2 b2 = bound_two(W.cw, W.c0[m], W.c1[m], xm, ym, zm, 1.5155444f, 1.7320508f + ps.walk_margin, g, mi);
-          cls = b2.fmax1 < 0.999f ? 0 : (b2.fmin1 > 1.001f ? 1 : 2);
-          need = b2.fmax2 >= 0.999f;
-        } else if (cls == 1) {
-          need = true;
-        } else {
-          need = bound_at(W.cw, W.c0[m], W.c1[m], xm, ym, zm, 1.7320508f + ps.walk_margin, g, mi).fmax >= 0.999f;
-        }
-        W.mcls[m][mb] = (unsigned char)(cls | (need ? 4 : 0));
+        const Bound2 b2 = mi ? pair_bound<true, true>(W.cw, W.q0[m], W.q1[m], xm, ym, zm, 1.5155444f, hw, g)
+                             : pair_bound<false, true>(W.cw, W.q0[m], W.q1[m], xm, ym, zm, 1.5155444f, hw, g);
+        const int cls = b2.fmax1 < 0.999f ? 0 : (b2.fmin1 > 1.001f ? 1 : 2);
+        W.mcls[m][mb] = (unsigned char)(cls | (b2.fmax2 >= 0.999f ? 4 : 0));
       }
       __syncwarp();
-      bool n0 = false, n1 = false;
-      for (int m = 0; m < n; ++m) {
-        n0 |= (W.mcls[m][lane] & 4) != 0;
-        n1 |= (W.mcls[m][lane + 32] & 4) != 0;
+      // per mini-brick: the walkers' bit, and its cells' common solid word or a place in the list
+      unsigned wm[2] = {0u, 0u};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = lane + 32 * h, mb = mb0 + k;
+        bool need = false, listed = false;
+        if (k < K) {
+          int own = 0x7fffffff;
+          for (int m = 0; m < n; ++m) {
+            const int mc = W.mcls[m][mb];
+            need |= (mc & 4) != 0;
+            listed |= (mc & 3) == 2;
+            if ((mc & 3) == 1) own = min(own, W.p[m]);
+          }
+          listed = listed && bi * BRICK + 2 * (mb & 3) < g.n[0] && bj * BRICK + 2 * ((mb >> 2) & 3) < g.n[1] &&
+                   bk * BRICK + 2 * (mb >> 4) < g.n[2];
+          W.val[mb] = listed ? (uint16_t)RW_LISTED : own != 0x7fffffff ? (uint16_t)(64 | (own << 7)) : (uint16_t)0;
+        }
+        wm[h] = __ballot_sync(full, need);
+        const unsigned bl = __ballot_sync(full, listed);
+        if (listed) W.list[nlisted + __popc(bl & ((1u << lane) - 1u))] = (unsigned char)mb;
+        nlisted += __popc(bl);
       }
-      const unsigned lo = __ballot_sync(full, n0), hi = __ballot_sync(full, n1);
-      if (lane == 0) bs.wmask[b] = ((unsigned long long)hi << 32) | lo;
+      if (lane == 0 && part == 0) {   // the slice's K mask bits
+        unsigned char* dst = reinterpret_cast<unsigned char*>(bs.wmask + b) + slice * (K >> 3);
+        if (slog == 0) *reinterpret_cast<unsigned long long*>(dst) = ((unsigned long long)wm[1] << 32) | wm[0];
+        else if (slog == 1) *reinterpret_cast<uint32_t*>(dst) = wm[0];
+        else if (slog == 2) *reinterpret_cast<uint16_t*>(dst) = (uint16_t)wm[0];
+        else *dst = (unsigned char)wm[0];
+      }
+      __syncwarp();
+      // cells of the other mini-bricks: two cells of one mini-brick (x, x + 1) per lane
+      if (A.cells && part == 0) {
+        const int ly0 = 2 * ((mb0 >> 2) & 3), lz0 = 2 * (mb0 >> 4);
+        for (int t = lane; t < 4 * K; t += 32) {
+          const int r = t >> 2, ly = ly0 + (r & (rows_y - 1)), lz = lz0 + r / rows_y;
+          const uint16_t v = W.val[(t & 3) + 4 * (ly >> 1) + 16 * (lz >> 1)];
+          const int i = bi * BRICK + 2 * (t & 3), j = bj * BRICK + ly, k = bk * BRICK + lz;
+          if (v == RW_LISTED || i >= g.n[0] || j >= g.n[1] || k >= g.n[2]) continue;
+          const uint32_t cell = ((uint32_t)k * g.n[1] + j) * g.n[0] + i;
+          if (i + 1 < g.n[0] && !(cell & 1u)) {
+            *reinterpret_cast<uint32_t*>(solid + cell) = (uint32_t)v | ((uint32_t)v << 16);
+          } else {
+            solid[cell] = v;
+            if (i + 1 < g.n[0]) solid[cell + 1] = v;
+          }
+        }
+      }
     } else {
-      if (lane == 0) {
+      if (lane == 0 && slice == 0 && part == 0) {
         bs.wmask[b] = ~0ull;   // every walker of this brick is tested
         if (over) atomicAdd(&status[ST_BRICK_OVERFLOW], 1ull);
       }
+      for (int k = lane; k < K; k += 32) W.list[k] = (unsigned char)(mb0 + k);
+      nlisted = K;
+      __syncwarp();
     }
-    // 3. cells, 32 per round
-    for (int r = 0; A.cells && r < (BRICK * BRICK * BRICK) / 32; ++r) {
-      const int cl = r * 32 + lane;
-      const int lx = cl & 7, ly = (cl >> 3) & 7, lz = cl >> 6;
+    // 3. cells of this part's listed mini-bricks, 32 per round (lane: mini-brick lane / 8, its cell
+    // lane & 7)
+    for (int r = part; A.cells && r < nlisted; r += 4 * parts) {
+      const int at = r + (lane >> 3) * parts;
+      const bool have = at < nlisted;
+      const int mb = have ? W.list[at] : 0;
+      const int lx = 2 * (mb & 3) + (lane & 1), ly = 2 * ((mb >> 2) & 3) + ((lane >> 1) & 1), lz = 2 * (mb >> 4) + ((lane >> 2) & 1);
       const int i = bi * BRICK + lx, j = bj * BRICK + ly, k = bk * BRICK + lz;
-      const bool in_dom = i < g.n[0] && j < g.n[1] && k < g.n[2];
-      const int mb = (lx >> 1) + 4 * (ly >> 1) + 16 * (lz >> 1);
+      const bool in_dom = have && i < g.n[0] && j < g.n[1] && k < g.n[2];
+      const float xi = (float)i, yj = (float)j, zk = (float)k;
       uint64_t any = 0ull;
       int best = 0, bestp = -1;
       unsigned pend = 0u;
       const int ncand = staged ? n : (over ? ps.P : (int)nc);
       for (int m = 0; in_dom && m < ncand; ++m) {
-        int pp, cls = 2, c0, c1;
-        const float4* cw;
-        bool cmi = mi;
+        int pp;
+        uint64_t mk;
         if (staged) {
-          pp = W.p[m]; cls = W.mcls[m][mb] & 3; cw = W.cw; c0 = W.c0[m]; c1 = W.c1[m];
+          pp = W.p[m];
+          const int cls = W.mcls[m][mb] & 3;
+          if (cls == 0) continue;
+          if (cls == 2) {
+            const Bound2 cb = mi ? pair_bound<true, false>(W.cw, W.q0[m], W.q1[m], xi + 0.5f, yj + 0.5f, zk + 0.5f, 0.649519053f, 0.0f, g)
+                                 : pair_bound<false, false>(W.cw, W.q0[m], W.q1[m], xi + 0.5f, yj + 0.5f, zk + 0.5f, 0.649519053f, 0.0f, g);
+            if (cb.fmax1 < 0.999f) continue;
+            if (!(cb.fmin1 > 1.001f)) {
+              pend |= 1u << m;   // the whole warp evaluates it below
+              continue;
+            }
+          }
+          mk = ~0ull;
         } else {
           if (over) pp = m;
           else {
@@ -616,56 +675,36 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A) {
             if (!(cid & 0x8000)) continue;
             pp = cid & 0x7fff;
           }
-          cw = bs.cworld; c0 = ps.desc[pp].c0; c1 = ps.desc[pp].c1; cmi = true;
-        }
-        if (cls == 0) continue;
-        uint64_t mk;
-        if (cls == 1) {
-          mk = ~0ull;
-        } else {
-          const CellBound cb = bound_at(cw, c0, c1, (float)i + 0.5f, (float)j + 0.5f, (float)k + 0.5f, 0.649519053f, g, cmi);
+          const int c0 = ps.desc[pp].c0, c1 = ps.desc[pp].c1;
+          const CellBound cb = bound_at(bs.cworld, c0, c1, xi + 0.5f, yj + 0.5f, zk + 0.5f, 0.649519053f, g);
           if (cb.fmax < 0.999f) continue;
-          if (cb.fmin > 1.001f) {
-            mk = ~0ull;
-          } else if (staged) {
-            pend |= 1u << m;   // the whole warp evaluates it below
-            continue;
-          } else {
-            mk = particle_mask_serial(cw, c0, c1, true, bs.cworld, c0, c1, i, j, k, g);
-          }
+          mk = cb.fmin > 1.001f ? ~0ull : particle_mask_serial(bs.cworld, c0, c1, i, j, k, g);
         }
         const int np = __popcll(mk);
         any |= mk;
         if (np > 0 && (np > best || (np == best && pp < bestp))) { best = np; bestp = pp; }
       }
       // the warp evaluates each straddling (cell, candidate) pair: 2 x 32 sub-samples
-      unsigned lanes_p = __ballot_sync(full, pend != 0u);
-      while (lanes_p) {
-        const int src = __ffs(lanes_p) - 1;
-        const unsigned pm = __shfl_sync(full, pend, src);
-        const int m = __ffs(pm) - 1;
-        const int scl = __shfl_sync(full, cl, src);
-        const int si = bi * BRICK + (scl & 7), sj = bj * BRICK + ((scl >> 3) & 7), sk = bk * BRICK + (scl >> 6);
-        const int e0 = W.e0[m], e1 = e0 + (W.c1[m] - W.c0[m]);
-        bool in_lo, in_hi;
-        const float sx = (float)si + 0.125f, sy = (float)sj + 0.125f, sz = (float)sk + 0.125f;
-        const float ax = 0.25f * (float)(lane & 3), ay = 0.25f * (float)((lane >> 2) & 3), az = 0.25f * (float)(lane >> 4);
-        if (mi)
-          subsample_pair_t<true>(W.cw, W.c0[m], W.c1[m], bs.cworld, e0, e1, sx + ax, sy + ay, sz + az, g, in_lo, in_hi);
-        else
-          subsample_pair_t<false>(W.cw, W.c0[m], W.c1[m], bs.cworld, e0, e1, sx + ax, sy + ay, sz + az, g, in_lo, in_hi);
-        const unsigned blo = __ballot_sync(full, in_lo);
-        const unsigned bhi = __ballot_sync(full, in_hi);
-        if (lane == src) {
-          const uint64_t mk = ((uint64_t)bhi << 32) | blo;
-          const int np = __popcll(mk);
-          const int pp = W.p[m];
-          any |= mk;
-          if (np > 0 && (np > best || (np == best && pp < bestp))) { best = np; bestp = pp; }
-          pend &= ~(1u << m);
+      for (int m = 0; staged && m < n; ++m) {
+        unsigned lanes_p = __ballot_sync(full, (pend >> m) & 1u);
+        queued += __popc(lanes_p);
+        while (lanes_p) {
+          const int src = __ffs(lanes_p) - 1;
+          lanes_p &= lanes_p - 1u;
+          const float sx = __shfl_sync(full, xi, src) + ax, sy = __shfl_sync(full, yj, src) + ay,
+                      sz = __shfl_sync(full, zk, src) + az;
+          bool in_lo, in_hi;
+          if (mi) subsample_pair<true>(W.cw, W.q0[m], W.q1[m], bs.cworld, W.e0[m], W.e1[m], sx, sy, sz, g, in_lo, in_hi);
+          else subsample_pair<false>(W.cw, W.q0[m], W.q1[m], bs.cworld, W.e0[m], W.e1[m], sx, sy, sz, g, in_lo, in_hi);
+          const unsigned blo = __ballot_sync(full, in_lo);
+          const unsigned bhi = __ballot_sync(full, in_hi);
+          if (lane == src) {
+            any |= ((uint64_t)bhi << 32) | blo;
+            const int np = __popc(blo) + __popc(bhi);
+            const int pp = W.p[m];
+            if (np > 0 && (np > best || (np == best && pp < bestp))) { best = np; bestp = pp; }
+          }
         }
-        ++queued;
-        lanes_p = __ballot_sync(full, pend != 0u);
       }
       if (in_dom) {
         const int count = __popcll(any);
@@ -674,16 +713,17 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A) {
       }
     }
     __syncwarp();
-    if (lane == 0) li = atomicAdd(&bs.bword[nbrick + 1], 1u);
-    li = __shfl_sync(full, li, 0);
+    if (lane == 0) u = warps + atomicAdd(&bs.bword[nbrick + 1], 1u);
+    u = __shfl_sync(full, u, 0);
   }
   if (lane == 0 && queued) atomicAdd(&status[ST_RASTER_QUEUED], queued);
 }
 
-__global__ void __launch_bounds__(256, 4) raster_kernel(const RasterArgs a) { raster_body(a); }
+__global__ void __launch_bounds__(256, 4) raster_kernel(const RasterArgs a) { raster_body(a, blockIdx.x, gridDim.x); }
 __global__ void __launch_bounds__(256, 4) raster_batched(const RasterArgs* __restrict__ args,
                                                          const BlockMap* __restrict__ map) {
-  raster_body(args[map[blockIdx.x].domain]);   // warps take the domain's bricks from its counter
+  const BlockMap m = map[blockIdx.x];
+  raster_body(args[m.domain], m.block, m.blocks);
 }
 
 // two blocks per SM: the raster runs beside the LBM, which takes the rest of each SM (four
