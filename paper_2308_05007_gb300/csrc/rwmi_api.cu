@@ -509,8 +509,9 @@ static bool fused_storage(int storage) { return storage == RWMI_STORE_FP32_SHIFT
 // raster of t+1 writes solid/wmask[(t+1) & 1], and bricks of t+1 are bricks[(t+1) & 1].
 // Schedules (cfg.overlap; rwmi_step_timed always takes 0 so that each phase is timed alone):
 //   0  one stream: LBM(t), poses(t+1), raster(t+1), walkers(t), sort/moments.
-//   1  poses(t+1) first; raster(t+1) on the side stream while LBM(t) runs on the main one (the
-//      raster is ALU-bound, the LBM HBM-bound); join; walkers on the main stream.
+//   1  poses(t+1) first; then raster(t+1), and LBM(t) beside it as soon as the raster's blocks are
+//      resident (the raster is ALU-bound, the LBM HBM-bound; with IBB or the staged update the
+//      raster runs on the side stream instead); walkers on the main stream.
 //   2  as 1, and the walkers (with sort and moments) run on their own stream, one step behind
 //      the fluid: walkers(t) overlap LBM(t+1) and raster(t+2). Step t+2's fluid work waits for
 //      walkers(t), the last reader of the parity it overwrites.
@@ -542,7 +543,7 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     phase_end(c, RWMI_PHASE_POSE);
   };
   const bool ibb = c->cfg.coupling == 1 && c->P > 0;
-  auto lbm = [&]() {    // LBM at t
+  auto lbm = [&](bool after_raster = false) {    // LBM at t
     phase_begin(c, RWMI_PHASE_LBM);
     IbbArgs ia;
     if (ibb) {   // node classes of t, refilling of nodes uncovered since t - 1
@@ -573,7 +574,8 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     if (!staged || reduce)
       launch_lbm(c->cfg.q, c->cfg.storage, reduce, c->g, c->f[c->fcur], c->f[c->fcur ^ 1], c->u[tp], c->solid[tp],
                  brick_set(c, tp), c->tau, c->cfg.rho0, c->acc[tp] + 6 * c->P, c->acc[tp],
-                 c->status, c->stream, c->cfg.lbm_block, ibb ? &ia : nullptr, dem || (reduce && !staged), !staged);
+                 c->status, c->stream, c->cfg.lbm_block, ibb ? &ia : nullptr, dem || (reduce && !staged), !staged,
+                 after_raster && !staged);
     // staged: the TMA update, plus the reduce-only pass on reduction steps; otherwise one pass,
     // or the update and the reduce-only pass for storages without the fused one (free DEM runs
     // only with storages that have it)
@@ -595,6 +597,14 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->stream, !ibb);
     c->launches++;
     phase_end(c, RWMI_PHASE_RASTER);
+  } else if (fork_raster && !ibb && !(c->tma_ok && c->cfg.lbm_staging)) {
+    // the raster first, then the update as soon as the raster's blocks are resident: on two streams
+    // the update sometimes took every SM first, and the raster ran only as it drained (256^3: 707
+    // to 768 us per step from one build to the next, 708 us in this order)
+    pose();
+    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->stream, true);
+    c->launches++;
+    lbm(true);
   } else if (fork_raster) {
     pose();
     cudaEventRecord(c->fork_ev, c->stream);

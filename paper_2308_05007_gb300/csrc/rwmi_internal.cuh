@@ -300,10 +300,13 @@ void launch_lbm_tma(int q, int storage, const CUtensorMap& map, const Geom& g, c
 // fused: the update and the reduction in one pass (binary32-shifted and binary64 storage; the
 // reduction steps of every run, and every step of free-DEM runs, which read the forces each
 // step). Its update stores the same bits as the plain update's.
+// after_raster: the launch before it on st is the raster of the next time, which the update shares
+// nothing with; the update starts as soon as the raster's blocks are resident, and ends after it.
 void launch_lbm(int q, int storage, bool reduce, const Geom& g, const void* fin, void* fout,
                 float* u, const uint16_t* solid, BrickSet bs, double tau, double rho0,
                 double* red, double* forces, unsigned long long* status, cudaStream_t st,
-                int block = 256, const IbbArgs* ibb = nullptr, bool fused = false, bool update = true);
+                int block = 256, const IbbArgs* ibb = nullptr, bool fused = false, bool update = true,
+                bool after_raster = false);
 
 // Free DEM (Section 2.2, Eqs. 4-11) of a context: contact law, state and per-pair memory. Pair
 // slots (i < j) sit at i P + j, wall slots (particle p, face 2 axis + side) at 6 p + face.

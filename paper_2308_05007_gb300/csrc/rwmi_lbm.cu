@@ -607,6 +607,9 @@ lbm_kernel(Geom g, Planes<Q, typename Store<STORE>::T> pl, float4* __restrict__ 
            const typename Store<STORE>::R* __restrict__ ib_g, int ib_cap) {
   lbm_body<Q, STORE, WALLS, MODE, IBB>(g, pl, u4, solid, bword, pose, posed, sp, tau, omega, guo0, rho0, red, forces,
                                        nodes, uprev, desc, cworld, ib_base, ib_word, ib_q, ib_g, ib_cap, blockIdx.x);
+  // launched behind the raster (launch_lbm's after_raster): one block outlasts it, so that whatever
+  // follows this kernel on the stream follows the raster too (returns at once otherwise)
+  if (blockIdx.x == gridDim.x - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // One launch over the cells of many domains: block -> (domain, block of that domain's grid). Its
@@ -821,10 +824,27 @@ void launch_ibb_links(int q, int storage, const Geom& g, BrickSet bs, const uint
 #undef RWMI_IBB_LINKS
 }
 
+// Launch of one kernel; with `overlap` it may start once every block of the kernel before it on the
+// stream has called griddepcontrol.launch_dependents or ended (programmatic dependent launch).
+template <typename... P, typename... A>
+static void launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, bool overlap, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 template <int Q, int STORE, bool IBB>
 static void launch_lbm_q(bool walls, bool reduce, const Geom& g, const void* fin, void* fout, float* u,
                          const uint16_t* solid, BrickSet bs, double tau, double rho0, double* red,
-                         double* forces, cudaStream_t st, int bsz, const IbbArgs& ib, bool fused, bool update) {
+                         double* forces, cudaStream_t st, int bsz, const IbbArgs& ib, bool fused, bool update,
+                         bool after_raster) {
   using T = typename Store<STORE>::T;
   using R = typename Store<STORE>::R;
   Planes<Q, T> pl;
@@ -837,16 +857,16 @@ static void launch_lbm_q(bool walls, bool reduce, const Geom& g, const void* fin
 #define RWMI_LBM_ARGS g, pl, reinterpret_cast<float4*>(u), solid, bs.bword, bs.pose, bs.posed, bs.sp, (R)tau, (R)(1.0 / tau), (R)(1.0 - 0.5 / tau), (R)rho0, red, forces, ib.nodes, ib.uprev, ib.desc, bs.cworld, ib.base, ib.word, ib.q, static_cast<const R*>(ib.g), ib.cap
   if constexpr (STORE == 1 || STORE == 3) {   // the fused mode of free-DEM runs
     if (fused) {
-      if (walls) lbm_kernel<Q, STORE, true, 2, IBB><<<grid, block, 0, st>>>(RWMI_LBM_ARGS);
-      else lbm_kernel<Q, STORE, false, 2, IBB><<<grid, block, 0, st>>>(RWMI_LBM_ARGS);
+      if (walls) launch_kernel(lbm_kernel<Q, STORE, true, 2, IBB>, grid, block, st, after_raster, RWMI_LBM_ARGS);
+      else launch_kernel(lbm_kernel<Q, STORE, false, 2, IBB>, grid, block, st, after_raster, RWMI_LBM_ARGS);
       return;
     }
   }
   if (walls) {
-    if (update) lbm_kernel<Q, STORE, true, 0, IBB><<<grid, block, 0, st>>>(RWMI_LBM_ARGS);
+    if (update) launch_kernel(lbm_kernel<Q, STORE, true, 0, IBB>, grid, block, st, after_raster, RWMI_LBM_ARGS);
     if (reduce) lbm_kernel<Q, STORE, true, 1, IBB><<<grid, block, 0, st>>>(RWMI_LBM_ARGS);
   } else {
-    if (update) lbm_kernel<Q, STORE, false, 0, IBB><<<grid, block, 0, st>>>(RWMI_LBM_ARGS);
+    if (update) launch_kernel(lbm_kernel<Q, STORE, false, 0, IBB>, grid, block, st, after_raster, RWMI_LBM_ARGS);
     if (reduce) lbm_kernel<Q, STORE, false, 1, IBB><<<grid, block, 0, st>>>(RWMI_LBM_ARGS);
   }
 #undef RWMI_LBM_ARGS
@@ -855,7 +875,7 @@ static void launch_lbm_q(bool walls, bool reduce, const Geom& g, const void* fin
 void launch_lbm(int q, int storage, bool reduce, const Geom& g, const void* fin, void* fout,
                 float* u, const uint16_t* solid, BrickSet bs, double tau, double rho0, double* red,
                 double* forces, unsigned long long* status, cudaStream_t st, int block, const IbbArgs* ibb,
-                bool fused, bool update) {
+                bool fused, bool update, bool after_raster) {
   (void)status;
   const bool walls = g.wall[0] || g.wall[1] || g.wall[2];
   const IbbArgs none{};
@@ -863,9 +883,9 @@ void launch_lbm(int q, int storage, bool reduce, const Geom& g, const void* fin,
   // IBB is built for binary32-shifted and binary64 storage (the configuration check refuses the
   // others); the other storages run the partially saturated cells only
 #define RWMI_LBM_PSM(QQ, SS) \
-  launch_lbm_q<QQ, SS, false>(walls, reduce, g, fin, fout, u, solid, bs, tau, rho0, red, forces, st, block, ib, fused, update)
+  launch_lbm_q<QQ, SS, false>(walls, reduce, g, fin, fout, u, solid, bs, tau, rho0, red, forces, st, block, ib, fused, update, after_raster)
 #define RWMI_LBM_CASE(QQ, SS)                                                                           \
-  if (ibb) launch_lbm_q<QQ, SS, true>(walls, reduce, g, fin, fout, u, solid, bs, tau, rho0, red, forces, st, block, ib, fused, update); \
+  if (ibb) launch_lbm_q<QQ, SS, true>(walls, reduce, g, fin, fout, u, solid, bs, tau, rho0, red, forces, st, block, ib, fused, update, after_raster); \
   else RWMI_LBM_PSM(QQ, SS)
   if (q == 15) {
     if (storage == 0) { RWMI_LBM_PSM(15, 0); }
