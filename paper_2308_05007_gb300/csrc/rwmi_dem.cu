@@ -7,15 +7,16 @@
 // switched off the trajectories then follow the CPU oracle's bit for bit, which the GPU tests
 // check; the formulas and their readings are the oracle's.
 //
-// One DEM step is two launches (or, for up to 128 particles, every DEM step of an LBM step is one
-// single-block launch, dem_fused_kernel, with block barriers between the two phases):
+// For up to 128 particles every DEM step of an LBM step is one launch of one thread-block cluster
+// (dem_cluster_kernel, cluster barriers between the two phases); beyond that a DEM step is two
+// launches:
 //   dem_contacts_kernel   one thread per pair slot (i < j) and per wall slot (particle, face):
 //                         reach test, Newton-Raphson geometry, force law; writes the slot's
 //                         force and torques (zero when apart) and its spring and Newton point;
 //   dem_integrate_kernel  one thread per particle: sums its slots in a fixed order (pairs by
 //                         partner index, then faces), adds the fluid force and gravity, advances
 //                         velocity, origin, spin and orientation.
-// Kernels wait on nothing; the launches follow each other on one stream.
+// The launches follow each other on one stream.
 #include "rwmi_internal.cuh"
 
 namespace rwmi {
@@ -374,44 +375,19 @@ __global__ void dem_integrate_kernel(DemArgs a) {
   if (p < a.P) integrate_particle(a, p);
 }
 
-// Every DEM step of one LBM step in one block: contact slots, a block barrier, integration, a
-// block barrier. For small particle counts, where launch latency would dominate.
-constexpr int DEM_FUSED_THREADS = 512;
-constexpr int DEM_FUSED_MAX_P = 128;
-__global__ void __launch_bounds__(DEM_FUSED_THREADS, 1) dem_fused_kernel(DemArgs a, int npairs, int substeps) {
-  const int slots = npairs + 6 * a.P;
-  for (int s = 0; s < substeps; ++s) {
-    for (int k = threadIdx.x; k < slots; k += blockDim.x) {
-      if (k < npairs) {
-        int i = 0, rem = k;
-        while (rem >= a.P - 1 - i) { rem -= a.P - 1 - i; ++i; }
-        pair_slot(a, i, i + 1 + rem);
-      } else {
-        const int w = k - npairs;
-        wall_slot(a, w / 6, w % 6);
-      }
-    }
-    __syncthreads();
-    for (int p = threadIdx.x; p < a.P; p += blockDim.x) integrate_particle(a, p);
-    __syncthreads();
+// Force and torque of pair slot (p, j) added to particle p's sums.
+__device__ __forceinline__ void add_pair(const DemArgs& a, int p, int j, double F[3], double T[3]) {
+  if (j < p) {
+    const size_t pr = (size_t)j * a.P + p;
+    for (int e = 0; e < 3; ++e) { F[e] = F[e] - a.pF[3 * pr + e]; T[e] = T[e] + a.pTj[3 * pr + e]; }
+  } else {
+    const size_t pr = (size_t)p * a.P + j;
+    for (int e = 0; e < 3; ++e) { F[e] = F[e] + a.pF[3 * pr + e]; T[e] = T[e] + a.pTi[3 * pr + e]; }
   }
 }
 
-__device__ void integrate_particle(const DemArgs& a, int p) {
-  const int P = a.P;
-  double F[3] = {0.0, 0.0, 0.0}, T[3] = {0.0, 0.0, 0.0};
-  // slots not in contact hold no force: adding their zeros would change no bit, so they are skipped
-  for (int j = 0; j < P; ++j) {
-    if (j < p) {
-      const size_t pr = (size_t)j * P + p;
-      if (a.act[pr])
-        for (int e = 0; e < 3; ++e) { F[e] = F[e] - a.pF[3 * pr + e]; T[e] = T[e] + a.pTj[3 * pr + e]; }
-    } else if (j > p) {
-      const size_t pr = (size_t)p * P + j;
-      if (a.act[pr])
-        for (int e = 0; e < 3; ++e) { F[e] = F[e] + a.pF[3 * pr + e]; T[e] = T[e] + a.pTi[3 * pr + e]; }
-    }
-  }
+// Particle p by one DEM step from the sums F, T of its pair slots in contact.
+__device__ void advance_particle(const DemArgs& a, int p, double F[3], double T[3]) {
   for (int f = 0; f < 6; ++f)
     if (a.actw[6 * (size_t)p + f])
       for (int e = 0; e < 3; ++e) {
@@ -459,6 +435,518 @@ __device__ void integrate_particle(const DemArgs& a, int p) {
   const double nn = sqrt(nq[0] * nq[0] + nq[1] * nq[1] + nq[2] * nq[2] + nq[3] * nq[3]);
   for (int e = 0; e < 4; ++e) q[e] = nq[e] / nn;
   a.posf[p] = make_float4((float)st[0], (float)st[1], (float)st[2], a.desc[p].rb);
+}
+
+__device__ void integrate_particle(const DemArgs& a, int p) {
+  double F[3] = {0.0, 0.0, 0.0}, T[3] = {0.0, 0.0, 0.0};
+  // slots not in contact hold no force: adding their zeros would change no bit, so they are skipped
+  for (int j = 0; j < a.P; ++j)
+    if (j != p && a.act[j < p ? (size_t)j * a.P + p : (size_t)p * a.P + j]) add_pair(a, p, j, F, T);
+  advance_particle(a, p, F, T);
+}
+
+// ---- every DEM step of one LBM step in one thread-block cluster ------------------------------
+// A DEM step is chains of binary64 operations, and one such warp instruction holds its quarter
+// of an SM for 64 cycles whatever the warp's active lanes (measured, dependent or not), so the cost
+// is the number of binary64 instructions per warp. One thread per slot and per particle (512
+// threads of one block) issued vector components, sums over control points, Hessian entries and
+// cofactors one after the other: 221 us per LBM step for 50 particles of a 120 x 120 x 180 box
+// with nothing in contact, about 600 us with its floor covered. Here the slots in reach are
+// compacted, a pair takes one warp (a half per particle), a face or a particle half a warp, with
+// lanes for the components of vectors and matrices, the control points, the ten sums of Eq. 3 and its
+// derivatives and the determinants; slots and particles spread over the SMs of a cluster. Every value
+// is formed by the same operations in the same order as in the functions above (sums over
+// control points by one lane in index order; x - y as x + (-y)), so the results are theirs bit for
+// bit.
+constexpr int DEM_CLUSTER = 8, DEM_THREADS = 256, DEM_WARPS = DEM_THREADS / 32;
+constexpr int DEM_FUSED_MAX_P = 128;
+
+struct HalfWarp {          // shared scratch of half a warp
+  double t[DEM_MAX_CP][6];  // per control point: k/r^2, its first and second derivative factors, r
+  double o[10];             // f, gradient, Hessian
+};
+
+// Where a half warp's lane finds itself: mask of the half's lanes, lane within it, the component e
+// it holds of a vector (lanes 0-2; the others repeat them), scratch; and the control point it holds
+// (n in all).
+struct Half {
+  unsigned mask;
+  int hl, e, n;
+  HalfWarp* s;
+  double c[3], k;
+};
+__device__ __forceinline__ double from(const Half& w, double v, int lane) { return __shfl_sync(w.mask, v, lane, 16); }
+__device__ __forceinline__ double comp3(const double* v, int e) { return e == 0 ? v[0] : e == 1 ? v[1] : v[2]; }
+__device__ __forceinline__ void gather3(const Half& w, double v, double out[3]) {
+  for (int e = 0; e < 3; ++e) out[e] = from(w, v, e);
+}
+// u . v of lane components
+__device__ __forceinline__ double lane_dot(const Half& w, double u, double v) {
+  double p[3];
+  gather3(w, u * v, p);
+  return p[0] + p[1] + p[2];
+}
+// component e of u x v
+__device__ __forceinline__ double lane_cross(const Half& w, double u, double v) {
+  const int e1 = w.e == 2 ? 0 : w.e + 1, e2 = w.e == 0 ? 2 : w.e - 1;
+  return from(w, u, e1) * from(w, v, e2) - from(w, u, e2) * from(w, v, e1);
+}
+// quat_matrix: lane 3 r + c < 9 forms R[r][c]
+__device__ __forceinline__ double lane_rotation(const Half& w, const double* q, int r, int c) {
+  const bool diag = r == c;
+  const int r1 = r == 2 ? 0 : r + 1, r2 = r == 0 ? 2 : r - 1;   // cyclic neighbours of the axis
+  const double m0 = q[1 + (diag ? r1 : r)], m1 = diag ? m0 : q[1 + c];
+  const double n0 = diag ? q[1 + r2] : q[0], n1 = diag ? n0 : q[1 + (3 - r - c)];
+  const double u = m0 * m1, v = n0 * n1;
+  const double two = 2.0 * (u + (!diag && c == r1 ? -v : v));
+  return diag ? 1.0 - two : two;
+}
+
+__device__ void half_points(const DemArgs& a, Half& w, int p, const double org[3]) {
+  const int l = w.hl < 9 ? w.hl : 0;
+  const double Rl = lane_rotation(w, a.st + 13 * p + 3, l / 3, l % 3);
+  const double z = a.zoom[p];
+  const ParticleDesc& d = a.desc[p];
+  w.n = min(d.c1 - d.c0, DEM_MAX_CP);
+  const float4 cb = w.hl < w.n ? a.cbody[d.c0 + w.hl] : make_float4(0.f, 0.f, 0.f, 0.f);
+  const double b[3] = {z * (double)cb.x, z * (double)cb.y, z * (double)cb.z};
+  for (int e = 0; e < 3; ++e)
+    w.c[e] = org[e] + from(w, Rl, 3 * e) * b[0] + from(w, Rl, 3 * e + 1) * b[1] + from(w, Rl, 3 * e + 2) * b[2];
+  w.k = z * z * (double)cb.w;
+}
+
+// mb_eval: lane i < n forms control point i's terms, lane m < 10 sums one of the ten results over
+// the points in order
+__device__ double half_eval(const Half& w, const double x[3], double g[3], double H[6]) {
+  HalfWarp& s = *w.s;
+  if (w.hl < w.n) {
+    const double r[3] = {x[0] - w.c[0], x[1] - w.c[1], x[2] - w.c[2]};
+    const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
+    const double inv2 = 1.0 / r2;
+    const double fi = w.k * inv2;
+    double* t = s.t[w.hl];
+    t[0] = fi;
+    t[1] = -2.0 * fi * inv2;
+    t[2] = 8.0 * fi * inv2 * inv2;
+    t[3] = r[0]; t[4] = r[1]; t[5] = r[2];
+  }
+  __syncwarp(w.mask);
+  const int m = w.hl;   // 0: f, 1-3: g, 4-6: H xx yy zz, 7-9: H xy xz yz
+  const int ia = m < 4 ? (m + 2) % 3 : m < 7 ? m - 4 : m < 9 ? 0 : 1, ib = m < 7 ? ia : m == 7 ? 1 : 2;
+  double acc = 0.0;
+  for (int i = 0; i < w.n; ++i) {
+    const double* t = s.t[i];
+    const double p = (m < 4 ? t[1] : t[2]) * t[3 + ia], p2 = p * t[3 + ib], d = t[1] + p2;
+    acc += m == 0 ? t[0] : m < 4 ? p : m < 7 ? d : p2;
+  }
+  if (m < 10) s.o[m] = acc;
+  __syncwarp(w.mask);
+  const double f = s.o[0];
+  for (int e = 0; e < 3; ++e) g[e] = s.o[1 + e];
+  for (int e = 0; e < 6; ++e) H[e] = s.o[4 + e];
+  __syncwarp(w.mask);
+  return f;
+}
+
+// solve3: lane q & 3 = 0 forms the determinant, 1-3 that with column q - 1 replaced by b; returns
+// lane e's component of the solution in d
+__device__ bool half_solve3(const Half& w, const double A[3][3], const double b[3], double& d) {
+  const int q = w.hl & 3;
+  double M[3][3];
+  for (int r = 0; r < 3; ++r)
+    for (int c = 0; c < 3; ++c) M[r][c] = c + 1 == q ? b[r] : A[r][c];
+  const double v = M[0][0] * (M[1][1] * M[2][2] - M[1][2] * M[2][1])
+                 - M[0][1] * (M[1][0] * M[2][2] - M[1][2] * M[2][0])
+                 + M[0][2] * (M[1][0] * M[2][1] - M[1][1] * M[2][0]);
+  const double det = from(w, v, 0);
+  if (!(fabs(det) > 1e-300)) return false;
+  d = from(w, v / det, w.e + 1);
+  return true;
+}
+
+// newton_update. Its length is compared as a square: the correctly rounded root of s exceeds 1 where
+// s > 1 + 2^-52, and 1e-12 where s > 0x1.357c299a88ea8p-80 (the largest double whose root does not).
+__device__ bool half_newton(const Half& w, const double A[3][3], const double G[3], double x[3]) {
+  const double b[3] = {-G[0], -G[1], -G[2]};
+  double d;
+  if (!half_solve3(w, A, b, d)) return false;
+  const double s = lane_dot(w, d, d);
+  double step = d;
+  if (s > 0x1.0000000000001p+0) step = 1.0 / sqrt(s) * d;
+  gather3(w, comp3(x, w.e) + step, x);
+  return s > 0x1.357c299a88ea8p-80;
+}
+
+__device__ void half_surface_along(const Half& w, const double xm[3], double xc[3]) {
+  double g[3], gx[3], H[6], x[3];
+  const double f = half_eval(w, xm, g, H);
+  const double xme = comp3(xm, w.e), ge = comp3(g, w.e);
+  const double q1 = (1.0 - f) / lane_dot(w, ge, ge);
+  double lo = 0.0, hi = q1, q = q1;
+  bool inside = false;
+  for (int h = 0; h <= SURFACE_HALVINGS; ++h) {
+    gather3(w, xme + hi * ge, x);
+    if (half_eval(w, x, gx, H) >= 1.0) { inside = true; break; }
+    hi = 0.5 * hi;
+  }
+  if (inside) {
+    q = hi;
+    for (int it = 0; it < SURFACE_ITERS; ++it) {
+      gather3(w, xme + q * ge, x);
+      const double fx = half_eval(w, x, gx, H);
+      if (fx == 1.0) break;
+      if (fx > 1.0) hi = q; else lo = q;
+      const double dq = lane_dot(w, comp3(gx, w.e), ge);
+      double qn = fabs(dq) > 1e-300 ? q - (fx - 1.0) / dq : 0.5 * (lo + hi);
+      if (!(qn > lo && qn < hi)) qn = 0.5 * (lo + hi);
+      if (qn == q) break;
+      q = qn;
+    }
+  }
+  gather3(w, xme + q * ge, xc);
+}
+
+// point_velocity, lane components: v + w x (x - org) of particle p
+__device__ __forceinline__ double lane_point_velocity(const DemArgs& a, const Half& w, int p, double r) {
+  const double* st = a.st + 13 * p;
+  return st[7 + w.e] + lane_cross(w, st[10 + w.e], r);
+}
+
+// contact_force, lane components
+__device__ double lane_contact_force(const DemArgs& a, const Half& w, double delta, double n, double vi, double vj,
+                                     double& xi) {
+  const double vr = vj - vi;
+  const double vn = lane_dot(w, vr, n);
+  double Fn = a.kn * delta - a.etan * vn;
+  if (Fn < 0.0) Fn = 0.0;
+  const double vt = vr - vn * n;
+  const double xn = lane_dot(w, xi, n);
+  xi = (xi - xn * n) + vt * a.dt;
+  double Ft = a.kt * xi + a.etat * vt;
+  const double mag = sqrt(lane_dot(w, Ft, Ft));
+  const double lim = a.mus * Fn;
+  if (mag > lim) {
+    const double sc = lim / mag;
+    Ft = Ft * sc;
+    xi = a.kt > 0.0 ? (Ft - a.etat * vt) / a.kt : 0.0;
+  }
+  return Ft - Fn * n;
+}
+
+// pair_slot after its prefilter, by one warp (lanes 0-15: particle i, 16-31: particle j)
+__device__ void warp_pair_slot(const DemArgs& a, int i, int j, Half& w) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, h = lane >> 4;
+  const size_t pr = (size_t)i * a.P + j;
+  const double* si = a.st + 13 * i;
+  const double* sj = a.st + 13 * j;
+  const double sie = si[w.e];
+  double de = sj[w.e] - sie;   // minimum image of j's origin seen from i's
+  const int wall = w.e == 0 ? a.wall[0] : w.e == 1 ? a.wall[1] : a.wall[2];
+  const double len = (double)(w.e == 0 ? a.n[0] : w.e == 1 ? a.n[1] : a.n[2]);
+  if (!wall) de -= len * floor(de / len + 0.5);
+  const double oje = sie + de;
+  const double dd = oje - sie;
+  const double reach = (double)a.desc[i].rb + (double)a.desc[j].rb;
+  const bool near = !(lane_dot(w, dd, dd) >= reach * reach);
+  const bool cont = a.act[pr] != 0;
+  double xm[3] = {a.xm[3 * pr], a.xm[3 * pr + 1], a.xm[3 * pr + 2]};
+  double xi = a.xi[3 * pr + w.e];
+  double F = 0.0, Ti = 0.0, Tj = 0.0;
+  bool touch = false;
+  if (near) {
+    double org[3];
+    gather3(w, h ? oje : sie, org);
+    half_points(a, w, h ? j : i, org);
+    const int n0 = __shfl_sync(full, w.n, 0), n1 = __shfl_sync(full, w.n, 16);
+    if (!cont) {   // the closest pair of control points, weighted by radius (first in order on ties)
+      double best = INFINITY;
+      int at = 0x7fffffff;
+      const double rk = sqrt(w.k);
+      for (int base = 0; base < n0 * n1; base += 32) {
+        const int l = base + lane, ia = min(l / n1, n0 - 1), ib = l - (l / n1) * n1;
+        double d[3];
+        for (int e = 0; e < 3; ++e) d[e] = __shfl_sync(full, w.c[e], 16 + ib) - __shfl_sync(full, w.c[e], ia);
+        const double gap = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) - __shfl_sync(full, rk, ia) -
+                           __shfl_sync(full, rk, 16 + ib);
+        if (l < n0 * n1 && gap < best) { best = gap; at = l; }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(full, best, o);
+        const int oa = __shfl_xor_sync(full, at, o);
+        if (ob < best || (ob == best && oa < at)) { best = ob; at = oa; }
+      }
+      if (at == 0x7fffffff) at = 0;
+      const int ba = at / n1, bb = 16 + at - ba * n1;
+      const double ra = __shfl_sync(full, rk, ba), rb = __shfl_sync(full, rk, bb), wr = ra / (ra + rb);
+      for (int e = 0; e < 3; ++e) {
+        const double ca = __shfl_sync(full, w.c[e], ba), cb = __shfl_sync(full, w.c[e], bb);
+        xm[e] = ca + wr * (cb - ca);
+      }
+    }
+    const int iters = cont ? NEWTON_CONT : NEWTON_NEW;
+    for (int it = 0; it < iters; ++it) {
+      double g[3], H[6], G[3], S[6];
+      half_eval(w, xm, g, H);
+      for (int e = 0; e < 3; ++e) G[e] = g[e] + __shfl_xor_sync(full, g[e], 16);
+      for (int e = 0; e < 6; ++e) S[e] = H[e] + __shfl_xor_sync(full, H[e], 16);
+      const double A[3][3] = {{S[0], S[3], S[4]}, {S[3], S[1], S[5]}, {S[4], S[5], S[2]}};
+      if (!half_newton(w, A, G, xm)) break;   // the same in both halves
+    }
+    double xc[3];
+    half_surface_along(w, xm, xc);
+    __syncwarp();
+    const double xc0 = __shfl_sync(full, comp3(xc, w.e), w.e), d = __shfl_sync(full, comp3(xc, w.e), 16 + w.e) - xc0;
+    const double dist = sqrt(lane_dot(w, d, d));
+    const double Rs0 = a.Rs[i], Rs1 = a.Rs[j];
+    const double delta = Rs0 + Rs1 - dist;
+    touch = delta > 0.0;
+    if (touch) {
+      const double nrm = dist > 0.0 ? d / dist : 0.0;
+      const double xcp = xc0 + (Rs0 - 0.5 * delta) * nrm;
+      const double ri = xcp - sie, rj = xcp - oje;
+      const double vi = lane_point_velocity(a, w, i, ri), vj = lane_point_velocity(a, w, j, rj);
+      F = lane_contact_force(a, w, delta, nrm, vi, vj, xi);
+      Ti = lane_cross(w, ri, F);
+      Tj = lane_cross(w, rj, -F);
+    }
+  }
+  __syncwarp();
+  if (lane == 0) a.act[pr] = touch ? 1 : 0;
+  if (lane < 3) {
+    if (near) a.xm[3 * pr + lane] = comp3(xm, lane);
+    a.xi[3 * pr + lane] = touch ? xi : 0.0;
+    a.pF[3 * pr + lane] = F;
+    a.pTi[3 * pr + lane] = Ti;
+    a.pTj[3 * pr + lane] = Tj;
+  }
+}
+
+// wall_slot after its prefilter, by half a warp: particle p, face f = 2 axis + side
+__device__ void half_wall_slot(const DemArgs& a, int p, int f, Half& w) {
+  const size_t wi = 6 * (size_t)p + f;
+  const int ax = f >> 1, side = f & 1;
+  const double* sp = a.st + 13 * p;
+  const double L = (double)a.n[ax];
+  const double gap = side ? L - sp[ax] : sp[ax];
+  const bool near = a.wall[ax] && !(gap >= (double)a.desc[p].rb);
+  const bool cont = a.actw[wi] != 0;
+  double xm[3] = {a.xmw[3 * wi], a.xmw[3 * wi + 1], a.xmw[3 * wi + 2]};
+  double xi = a.xiw[3 * wi + w.e];
+  double F = 0.0, T = 0.0;
+  bool touch = false;
+  if (near) {
+    half_points(a, w, p, sp);
+    const double sg = side ? -1.0 : 1.0;
+    if (!cont) {   // the control point reaching closest to the face (first in order on ties)
+      const double rk = sqrt(w.k), ca = comp3(w.c, ax);
+      const double reach = side ? -(ca + rk) : ca - rk;
+      double best = INFINITY;
+      int bi = 0x7fffffff;
+      if (w.hl < w.n && reach < best) { best = reach; bi = w.hl; }
+      for (int o = 8; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(w.mask, best, o, 16);
+        const int oi = __shfl_xor_sync(w.mask, bi, o, 16);
+        if (ob < best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+      }
+      if (bi == 0x7fffffff) bi = 0;
+      const double rb = from(w, rk, bi);
+      for (int e = 0; e < 3; ++e) {
+        xm[e] = from(w, w.c[e], bi);
+        if (e == ax) xm[e] -= sg * rb;
+      }
+    }
+    const int iters = cont ? NEWTON_CONT : NEWTON_NEW;
+    for (int it = 0; it < iters; ++it) {
+      double g[3], H[6];
+      const double fx = half_eval(w, xm, g, H);
+      const double G[3] = {ax == 0 ? g[1] : g[0], ax == 2 ? g[1] : g[2], fx - 1.0};
+      // rows of the Hessian of the two axes along the face
+      const double A[3][3] = {{ax == 0 ? H[3] : H[0], ax == 0 ? H[1] : H[3], ax == 0 ? H[5] : H[4]},
+                              {ax == 2 ? H[3] : H[4], ax == 2 ? H[1] : H[5], ax == 2 ? H[5] : H[2]},
+                              {g[0], g[1], g[2]}};
+      if (!half_newton(w, A, G, xm)) break;
+    }
+    const double wall = side ? L : 0.0;
+    const double dist = (comp3(xm, ax) - wall) * sg;
+    const double delta = a.Rs[p] - dist;
+    touch = delta > 0.0;
+    if (touch) {
+      const double nrm = w.e == ax ? sg : 0.0;
+      const double xcp = (w.e == ax ? wall : comp3(xm, w.e)) + 0.5 * delta * nrm;
+      const double r = xcp - sp[w.e];
+      const double vi = lane_point_velocity(a, w, p, r);
+      F = lane_contact_force(a, w, delta, -nrm, vi, 0.0, xi);
+      T = lane_cross(w, r, F);
+    }
+  }
+  __syncwarp(w.mask);
+  if (w.hl == 0) a.actw[wi] = touch ? 1 : 0;
+  if (w.hl < 3) {
+    if (near) a.xmw[3 * wi + w.hl] = comp3(xm, w.hl);
+    a.xiw[3 * wi + w.hl] = touch ? xi : 0.0;
+    a.wF[3 * wi + w.hl] = F;
+    a.wT[3 * wi + w.hl] = T;
+  }
+}
+
+// integrate_particle by half a warp: lanes 0-2 hold the force sums, 3-5 the torque sums
+__device__ void half_integrate(const DemArgs& a, int p, const unsigned char* partner, int np, const Half& w) {
+  const bool tor = w.hl >= 3 && w.hl < 6;
+  double S = 0.0;
+  for (int k = 0; k < np; ++k) {
+    const int j = partner[k];
+    const size_t at = 3 * (j < p ? (size_t)j * a.P + p : (size_t)p * a.P + j) + w.e;
+    const double v = tor ? (j < p ? a.pTj[at] : a.pTi[at]) : a.pF[at];
+    S = S + (!tor && j < p ? -v : v);
+  }
+  for (int f = 0; f < 6; ++f)
+    if (a.actw[6 * (size_t)p + f]) {
+      const size_t at = 3 * (6 * (size_t)p + f) + w.e;
+      S = S + (tor ? a.wT[at] : a.wF[at]);
+    }
+  const double m = a.mass[p], dt = a.dt;
+  if (a.Fe) S = S + a.Fe[6 * p + (tor ? 3 : 0) + w.e];
+  const double F = S + m * (w.e == 0 ? a.g[0] : w.e == 1 ? a.g[1] : a.g[2]);   // lanes 0-2
+  const double T = from(w, S, 3 + w.e);
+  double* st = a.st + 13 * p;
+  double q[4];
+  for (int e = 0; e < 4; ++e) q[e] = st[3 + e];
+  // translation: symplectic Euler
+  const double vel = st[7 + w.e] + dt * (F / m);
+  const double pos = st[w.e] + dt * vel;
+  // rotation: I_w = R I_b R^T, w += dt I_w^-1 (T - w x I_w w); lane 3 r + c < 9 holds entry (r, c)
+  const int l = w.hl < 9 ? w.hl : 0, r = l / 3, c = l - 3 * r;
+  const double R = lane_rotation(w, q, r, c);
+  const double* I6 = a.Ib + 6 * p;   // xx yy zz xy xz yz
+  const double I0 = I6[c == 0 ? 0 : 2 + c], I1 = I6[c == 0 ? 3 : c == 1 ? 1 : 5], I2 = I6[c == 2 ? 2 : 4 + c];
+  const double RI = from(w, R, 3 * r) * I0 + from(w, R, 3 * r + 1) * I1 + from(w, R, 3 * r + 2) * I2;
+  const double Iwl = from(w, RI, 3 * r) * from(w, R, 3 * c) + from(w, RI, 3 * r + 1) * from(w, R, 3 * c + 1) +
+                     from(w, RI, 3 * r + 2) * from(w, R, 3 * c + 2);
+  double Iw[3][3];
+  for (int e = 0; e < 9; ++e) Iw[e / 3][e % 3] = from(w, Iwl, e);
+  double spin = st[10 + w.e], ws[3];
+  gather3(w, spin, ws);
+  const double Lw = (w.e == 0 ? Iw[0][0] : w.e == 1 ? Iw[1][0] : Iw[2][0]) * ws[0] +
+                    (w.e == 0 ? Iw[0][1] : w.e == 1 ? Iw[1][1] : Iw[2][1]) * ws[1] +
+                    (w.e == 0 ? Iw[0][2] : w.e == 1 ? Iw[1][2] : Iw[2][2]) * ws[2];
+  double rhs[3], dw;
+  gather3(w, T - lane_cross(w, spin, Lw), rhs);
+  if (half_solve3(w, Iw, rhs, dw)) spin = spin + dt * dw;
+  gather3(w, spin, ws);
+  // orientation: q += dt/2 (0, w) q, normalised; lane 0: qw - h (w.q), lanes 1-3: q_e + h (qw w + w x q)_e
+  const double h = 0.5 * dt;
+  const int i = w.hl & 3, e0 = i == 0 ? 0 : i - 1, e1 = e0 == 2 ? 0 : e0 + 1, e2 = e0 == 0 ? 2 : e0 - 1;
+  const double m0 = i == 0 ? ws[0] * q[1] : q[0] * comp3(ws, e0);
+  const double m1 = comp3(ws, e1) * comp3(q + 1, i == 0 ? e1 : e2);   // i = 0: w1 q1; else w_{e1} q_{e2}
+  const double m2 = comp3(ws, e2) * comp3(q + 1, i == 0 ? e2 : e1);
+  const double t = i == 0 ? m0 + m1 : m1 + -m2;
+  const double u = i == 0 ? t + m2 : m0 + t;
+  const double hu = h * u;
+  const double nql = (i == 0 ? q[0] : comp3(q + 1, e0)) + (i == 0 ? -hu : hu);
+  const double sq = nql * nql;
+  const double nn = sqrt(from(w, sq, 0) + from(w, sq, 1) + from(w, sq, 2) + from(w, sq, 3));
+  const double qn = nql / nn;
+  __syncwarp(w.mask);   // the state has been read
+  if (w.hl < 3) {
+    st[w.hl] = pos;
+    st[7 + w.hl] = vel;
+    st[10 + w.hl] = spin;
+  }
+  if (w.hl < 4) st[3 + w.hl] = qn;
+  double o[3];
+  gather3(w, pos, o);
+  if (w.hl == 0) a.posf[p] = make_float4((float)o[0], (float)o[1], (float)o[2], a.desc[p].rb);
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+}
+
+__global__ void __cluster_dims__(DEM_CLUSTER, 1, 1) __launch_bounds__(DEM_THREADS, 1)
+dem_cluster_kernel(DemArgs a, int substeps) {
+  constexpr int MAX_LOCAL = (DEM_FUSED_MAX_P + DEM_CLUSTER - 1) / DEM_CLUSTER;
+  __shared__ HalfWarp s_half[2 * DEM_WARPS];
+  __shared__ uint16_t s_pairs[(DEM_FUSED_MAX_P * DEM_FUSED_MAX_P + DEM_CLUSTER - 1) / DEM_CLUSTER];
+  __shared__ uint16_t s_walls[(6 * DEM_FUSED_MAX_P + DEM_CLUSTER - 1) / DEM_CLUSTER];
+  __shared__ unsigned char s_partner[MAX_LOCAL][DEM_FUSED_MAX_P];
+  __shared__ int s_np, s_nw;
+  const int P = a.P, rank = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, half = lane >> 4;
+  Half w;
+  w.mask = 0xffffu << (16 * half);
+  w.hl = lane & 15;
+  w.e = w.hl % 3;
+  w.n = 0;
+  w.s = s_half + 2 * warp + half;
+  for (int step = 0; step < substeps; ++step) {
+    if (threadIdx.x == 0) { s_np = 0; s_nw = 0; }
+    __syncthreads();
+    // slots within binary32 reach (bound spheres apart by more than a margin cannot touch), dealt
+    // out to the blocks one by one; slots that left reach are cleared
+    for (int k = threadIdx.x * DEM_CLUSTER + rank; k < P * P + 6 * P; k += DEM_THREADS * DEM_CLUSTER) {
+      if (k < P * P) {
+        const int i = k / P, j = k - i * P;
+        if (i >= j) continue;
+        const float4 pi = a.posf[i], pj = a.posf[j];
+        const float dv[3] = {pj.x - pi.x, pj.y - pi.y, pj.z - pi.z};
+        float d2 = 0.0f;
+        for (int e = 0; e < 3; ++e) {
+          float dd = dv[e];
+          if (!a.wall[e]) dd -= (float)a.n[e] * rintf(dd / (float)a.n[e]);
+          d2 += dd * dd;
+        }
+        const float reach = pi.w + pj.w + 0.01f;
+        if (d2 > reach * reach) {
+          if (a.act[k]) { a.act[k] = 0; clear3(a.xi + 3 * (size_t)k); }
+        } else {
+          s_pairs[atomicAdd(&s_np, 1)] = (uint16_t)k;
+        }
+      } else {
+        const int wi = k - P * P, p = wi / 6, ax = (wi - 6 * p) >> 1, side = wi & 1;
+        const float4 pf = a.posf[p];
+        const float c = ax == 0 ? pf.x : ax == 1 ? pf.y : pf.z;
+        const float gapf = side ? (float)a.n[ax] - c : c;
+        if (!a.wall[ax] || gapf > pf.w + 0.01f) {
+          if (a.actw[wi]) { a.actw[wi] = 0; clear3(a.xiw + 3 * (size_t)wi); }
+        } else {
+          s_walls[atomicAdd(&s_nw, 1)] = (uint16_t)wi;
+        }
+      }
+    }
+    __syncthreads();
+    for (int k = warp; k < s_np; k += DEM_WARPS) {
+      const int pr = s_pairs[k];
+      warp_pair_slot(a, pr / P, pr % P, w);
+    }
+    // faces from the last warp on, so that they land beside the fewest pairs
+    for (int k = 2 * (DEM_WARPS - 1 - warp) + half; k < s_nw; k += 2 * DEM_WARPS) {
+      const int wi = s_walls[k];
+      half_wall_slot(a, wi / 6, wi % 6, w);
+    }
+    __syncwarp();   // the halves of a warp may have left the loop apart
+    cluster_barrier();
+    // this block's particles, two per warp: their partners in contact by index, then the integration
+    const int local = (P - rank + DEM_CLUSTER - 1) / DEM_CLUSTER;
+    for (int l0 = 2 * warp; l0 < local; l0 += 2 * DEM_WARPS) {
+      int np = 0;
+      for (int k = 0; k < 2 && l0 + k < local; ++k) {
+        const int p = (l0 + k) * DEM_CLUSTER + rank;
+        int n = 0;
+        for (int base = 0; base < P; base += 32) {
+          const int j = base + lane;
+          const bool on = j < P && j != p && a.act[j < p ? j * P + p : p * P + j];
+          const unsigned bal = __ballot_sync(0xffffffffu, on);
+          if (on) s_partner[l0 + k][n + __popc(bal & ((1u << lane) - 1u))] = (unsigned char)j;
+          n += __popc(bal);
+        }
+        if (half == k) np = n;
+      }
+      __syncwarp();
+      if (l0 + half < local) half_integrate(a, (l0 + half) * DEM_CLUSTER + rank, s_partner[l0 + half], np, w);
+      __syncwarp();
+    }
+    cluster_barrier();
+  }
 }
 
 // zoom s_p = 1 - R_s,p / R_c,p with R_c,p = max_i (|c_i| + sqrt(k_i)) over the body frame
@@ -567,8 +1055,8 @@ void launch_dem_init(const DemArgs& a, cudaStream_t st) {
 int launch_dem(const DemArgs& a, int substeps, cudaStream_t st) {
   if (a.P <= 0) return 0;
   const int npairs = a.P * (a.P - 1) / 2;
-  if (a.P <= DEM_FUSED_MAX_P) {   // one block takes every step
-    dem_fused_kernel<<<1, DEM_FUSED_THREADS, 0, st>>>(a, npairs, substeps);
+  if (a.P <= DEM_FUSED_MAX_P) {   // one cluster takes every step
+    dem_cluster_kernel<<<DEM_CLUSTER, DEM_THREADS, 0, st>>>(a, substeps);
     return 1;
   }
   const int slots = npairs + 6 * a.P;

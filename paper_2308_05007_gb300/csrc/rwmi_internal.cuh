@@ -331,7 +331,7 @@ struct DemArgs {
   double kn, etan, kt, etat, mus, g[3];
   double dt;                                   // 1 / substeps
 };
-// substeps DEM steps: one single-block launch for up to 128 particles, else two launches per DEM
+// substeps DEM steps: one launch of one cluster for up to 128 particles, else two launches per DEM
 // step (contacts, then integration); returns the number of launches
 int launch_dem(const DemArgs& a, int substeps, cudaStream_t st);
 // the zoom factors from the sphere radii (rwmi_set_dem)

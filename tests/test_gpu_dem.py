@@ -263,3 +263,34 @@ def test_ibb_schedules_and_graphs_agree():
             else:
                 for a, b in zip(ref, res):
                     assert np.array_equal(a, b), (overlap, graphs)
+
+
+@pytest.mark.parametrize("n_particles, dims, centres, steps", [
+    (1, (24, 24, 40), (1, 1), 160),      # one particle onto the floor: faces only
+    (2, (40, 36, 44), (16, 16), 60),     # as many control points as the DEM takes
+    (7, (52, 50, 60), (1, 5), 160),      # fewer particles than blocks in the cluster
+    (60, (84, 80, 76), (1, 3), 160),
+    (128, (100, 96, 92), (1, 3), 160),   # the most one cluster takes
+])
+def test_cluster_path_bit_exact(n_particles, dims, centres, steps):
+    """Up to 128 particles: every DEM step of an LBM step in one cluster launch, bit-identical to
+    the oracle (fluid force off) through pair and face contacts."""
+    from paper_2308_05007_gb300.rwmi import Simulation
+    w = I.dem_box(dims=dims, n_particles=1, seed=5, hydro=0, n_walkers=0, gravity=(0.0, 0.0, -1e-3))
+    mb = I.random_metaballs(np.random.default_rng(9), n_particles, dims, wall_mask=4, n_centers=centres, sigma=0.8,
+                            k_range=(1.5, 3.0))
+    aim = mb.origin.mean(0) - mb.origin   # pairs meet at the centre; fewer than 7 fall onto the floor
+    if n_particles < 7:
+        aim = aim - (0.0, 0.0, dims[2] / 2.0)
+    v = 0.12 * aim / np.linalg.norm(aim, axis=1, keepdims=True)
+    spin = np.random.default_rng(10).normal(scale=0.01, size=(n_particles, 3))
+    w = I.with_(w, metaballs=mb, dem=I.Dem(density=2.5, sphere_radius=I.sphere_radii(mb), velocity=v, spin=spin, kn=50.0,
+                                           eta_n=2.0, kt=20.0, eta_t=1.0, mu_s=0.4, gravity=(0.0, 0.0, -1e-3), hydro=0))
+    ora = Oracle.from_workload(w, seed_walkers=False)
+    with Simulation.from_workload(w, seed_walkers=False) as sim:
+        sim.step(steps)
+        ora.dem_advance(steps)
+        st = sim.particle_state()
+    np.testing.assert_array_equal(st, ora.particle_state())
+    free = v + steps * np.asarray(w.dem.gravity)
+    assert (np.abs(st[:, 7:10] - free).max(1) > 1e-6).any(), "no contact happened"
