@@ -379,8 +379,7 @@ rwmi_status build_current_frame(rwmi_ctx* c) {
     launch_clear_u32(c->bword[pp], c->nbrick + BWORD_EXTRA, c->stream);
     launch_pose_bin(c->g, particle_set(c), brick_set(c, pp), c->d_T, -1, c->cfg.body_force,
                     c->cfg.force_period, 1, c->acc[pp], c->cfg.q, c->tau, c->stream);
-    launch_nodes(c->cfg.q, c->cfg.storage, c->g, particle_set(c), brick_set(c, pp), c->node[pp], c->node[pp],
-                 c->f[c->fcur], c->cfg.rho0, false, c->stream);
+    launch_nodes(c->g, particle_set(c), brick_set(c, pp), c->node[pp], c->stream);
     c->launches += 3;
   }
   CK(cudaMemsetAsync(c->bword[par], 0, sizeof(uint32_t) * (c->nbrick + BWORD_EXTRA), c->stream));
@@ -388,7 +387,8 @@ rwmi_status build_current_frame(rwmi_ctx* c) {
                   c->cfg.force_period, 1, c->acc[par], c->cfg.q, c->tau, c->stream);
   c->launches++;
   if (c->P > 0) {
-    launch_raster(c->g, particle_set(c), brick_set(c, par), c->solid[par], c->status, c->nsm, c->stream);
+    launch_raster(c->g, particle_set(c), brick_set(c, par), c->solid[par], c->status, c->nsm, c->stream,
+                  c->cfg.coupling == 1 ? c->node[par] : nullptr);
     c->launches++;
   }
   CK(cudaGetLastError());
@@ -543,13 +543,17 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     phase_end(c, RWMI_PHASE_POSE);
   };
   const bool ibb = c->cfg.coupling == 1 && c->P > 0;
-  auto lbm = [&](bool after_raster = false) {    // LBM at t
+  uint16_t* classes = ibb ? c->node[tn] : nullptr;   // the raster of t+1 writes them
+  if (ibb) {   // refilling of nodes uncovered since t - 1, before the raster of t+1 takes their classes' place
     phase_begin(c, RWMI_PHASE_LBM);
+    launch_refill(c->cfg.q, c->cfg.storage, c->g, brick_set(c, tp), c->node[tn], c->node[tp], c->f[c->fcur],
+                  c->cfg.rho0, c->stream);
+    c->launches++;
+  }
+  auto lbm = [&](bool after_raster = false) {    // LBM at t
+    if (!ibb) phase_begin(c, RWMI_PHASE_LBM);
     IbbArgs ia;
-    if (ibb) {   // node classes of t, refilling of nodes uncovered since t - 1
-      launch_nodes(c->cfg.q, c->cfg.storage, c->g, ps, brick_set(c, tp), c->node[tn], c->node[tp],
-                   c->f[c->fcur], c->cfg.rho0, true, c->stream);
-      c->launches++;
+    if (ibb) {
       ia.nodes = c->node[tp];
       ia.uprev = reinterpret_cast<const float4*>(c->u[tn]);
       ia.desc = c->desc;
@@ -558,6 +562,7 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
       c->launches += 2;
       ia.base = c->ibl.base;
       ia.word = c->ibl.word;
+      ia.mask = c->wmask[tp];
       ia.q = c->ibl.q;
       ia.g = c->ibl.g;
       ia.cap = c->ibl.cap;
@@ -594,7 +599,7 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     lbm();
     pose();
     phase_begin(c, RWMI_PHASE_RASTER);
-    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->stream, !ibb);
+    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->stream, classes);
     c->launches++;
     phase_end(c, RWMI_PHASE_RASTER);
   } else if (fork_raster && !ibb && !(c->tma_ok && c->cfg.lbm_staging)) {
@@ -602,14 +607,14 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     // the update sometimes took every SM first, and the raster ran only as it drained (256^3: 707
     // to 768 us per step from one build to the next, 708 us in this order)
     pose();
-    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->stream, true);
+    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->stream);
     c->launches++;
     lbm(true);
   } else if (fork_raster) {
     pose();
     cudaEventRecord(c->fork_ev, c->stream);
     cudaStreamWaitEvent(c->side, c->fork_ev, 0);
-    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->side, !ibb);
+    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->side, classes);
     c->launches++;
     cudaEventRecord(c->join_ev, c->side);
     lbm();
@@ -619,7 +624,7 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     pose();
     phase_begin(c, RWMI_PHASE_RASTER);
     if (c->P > 0) {
-      launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->stream, !ibb);
+      launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->stream, classes);
       c->launches++;
     }
     phase_end(c, RWMI_PHASE_RASTER);
@@ -1242,8 +1247,7 @@ RWMI_API rwmi_status rwmi_autotune(rwmi_ctx* c, int32_t* chosen) try {
   IbbArgs ia;
   const bool ibb = c->cfg.coupling == 1 && c->P > 0;
   if (ibb) {   // node classes of this time (no refilling: the step itself redoes them)
-    launch_nodes(c->cfg.q, c->cfg.storage, c->g, particle_set(c), brick_set(c, tp), c->node[tp ^ 1], c->node[tp],
-                 c->f[c->fcur], c->cfg.rho0, false, c->stream);
+    launch_nodes(c->g, particle_set(c), brick_set(c, tp), c->node[tp], c->stream);
     c->launches++;
     ia.nodes = c->node[tp];
     ia.uprev = reinterpret_cast<const float4*>(c->u[tp ^ 1]);
@@ -1253,6 +1257,7 @@ RWMI_API rwmi_status rwmi_autotune(rwmi_ctx* c, int32_t* chosen) try {
     c->launches += 2;
     ia.base = c->ibl.base;
     ia.word = c->ibl.word;
+    ia.mask = c->wmask[tp];
     ia.q = c->ibl.q;
     ia.g = c->ibl.g;
     ia.cap = c->ibl.cap;
@@ -1473,7 +1478,7 @@ RWMI_API rwmi_status rwmi_solid(rwmi_ctx* c, int32_t* count, int32_t* owner) try
     // here, from its bricks (intact until the next step), by a full raster with a reset work
     // counter (it rewrites the same walker masks)
     CK(cudaMemsetAsync(c->bword[par] + c->nbrick + 1, 0, sizeof(uint32_t), c->stream));
-    launch_raster(c->g, particle_set(c), brick_set(c, par), c->solid[par], c->status, c->nsm, c->stream, true);
+    launch_raster(c->g, particle_set(c), brick_set(c, par), c->solid[par], c->status, c->nsm, c->stream);
     c->launches++;
   }
   launch_unpack_solid(c->g, c->solid[par], c->bword[par], tmp, tmp + c->ncell, c->stream);
@@ -1495,8 +1500,7 @@ RWMI_API rwmi_status rwmi_nodes(rwmi_ctx* c, int32_t* node) try {
   if (s != RWMI_OK) return s;
   uint16_t* tmp = (uint16_t*)c->scratch;
   if (c->P > 0) {
-    launch_nodes(c->cfg.q, c->cfg.storage, c->g, particle_set(c), brick_set(c, par), tmp, tmp, c->f[c->fcur],
-                 c->cfg.rho0, false, c->stream);
+    launch_nodes(c->g, particle_set(c), brick_set(c, par), tmp, c->stream);
     c->launches++;
   } else {
     CK(cudaMemsetAsync(tmp, 0, sizeof(uint16_t) * n, c->stream));

@@ -7,9 +7,9 @@
 //                     force/momentum accumulators
 //   raster_kernel     solid sub-sample count + owner for every cell of bricks that touch a
 //                     particle (Eq. 3, 4x4x4 sub-samples, binary32 decisions bit-identical to
-//                     the CPU oracle's)
-//   node_kernel       with the paper's coupling: solid/fluid node classes of the flagged bricks
-//                     and the refilling of nodes uncovered since the previous step (Eq. 27)
+//                     the CPU oracle's); with the paper's coupling the solid/fluid node classes
+//   refill_kernel     with the paper's coupling: node classes of the other bricks, refilling of
+//                     nodes uncovered since the previous step (Eq. 27)
 #include "rwmi_lattice.cuh"
 
 namespace rwmi {
@@ -356,6 +356,23 @@ __device__ __forceinline__ CellBound bound_at(const float4* cw, int c0, int c1, 
   return b;
 }
 
+// Is (x, y, z) inside particle [c0, c1) by Eq. 3 in the CPU oracle's binary32 sequence? A fast
+// value (fast reciprocal, contraction allowed; error ~1e-6 relative) decides outside 4e-5 of 1,
+// the exact sequence inside that band, so the answer always equals the exact one.
+__device__ __forceinline__ bool inside_exact(const float4* __restrict__ cw, int c0, int c1, float x, float y,
+                                             float z, const Geom& g) {
+  float f = 0.0f;
+  for (int i = c0; i < c1; ++i) {
+    const float4 c = cw[i];
+    const float dx = min_image_rn(x - c.x, (float)g.n[0], g.wall[0]);
+    const float dy = min_image_rn(y - c.y, (float)g.n[1], g.wall[1]);
+    const float dz = min_image_rn(z - c.z, (float)g.n[2], g.wall[2]);
+    f += __fdividef(c.w, dx * dx + dy * dy + dz * dz);
+  }
+  if (fabsf(f - 1.0f) > 4e-5f) return f >= 1.0f;
+  return metaball_exact(cw, c0, c1, x, y, z, g) >= 1.0f;
+}
+
 // Whole-cell mask evaluated by one thread from the wrapped control points (same bricks): the fast
 // value, and within 4e-5 of 1 the exact binary32 sequence. Bit s = a + 4 b + 16 c is sub-sample
 // (a, b, c) of cell (i, j, k).
@@ -439,6 +456,20 @@ __device__ __forceinline__ void subsample_pair(const float4* cw, int q0, int q1,
   in_hi = fabsf(fhi - 1.0f) > 4e-5f ? fhi >= 1.0f : metaball_exact(cw_exact, e0, e1, x, y, zh, g) >= 1.0f;
 }
 
+// Is the point (x, y, z) inside, likewise.
+template <bool MI>
+__device__ __forceinline__ bool point_inside(const float4* cw, int q0, int q1, const float4* cw_exact, int e0, int e1,
+                                             float x, float y, float z, const Geom& g) {
+  float f = 0.0f;
+  for (int q = q0; q < q1; ++q) {
+    const CenterPair c = load_pair(cw, q);
+    const float dx0 = disp<MI>(x, c.xy.x, 0, g), dx1 = disp<MI>(x, c.xy.y, 0, g), dy0 = disp<MI>(y, c.xy.z, 1, g),
+                dy1 = disp<MI>(y, c.xy.w, 1, g), dz0 = disp<MI>(z, c.zk.x, 2, g), dz1 = disp<MI>(z, c.zk.y, 2, g);
+    f = add_quotients(f, c.zk.z, dx0 * dx0 + dy0 * dy0 + dz0 * dz0, c.zk.w, dx1 * dx1 + dy1 * dy1 + dz1 * dz1);
+  }
+  return fabsf(f - 1.0f) > 4e-5f ? f >= 1.0f : metaball_exact(cw_exact, e0, e1, x, y, z, g) >= 1.0f;
+}
+
 constexpr int RW_WARPS = 8;        // warps (pieces in flight) per block
 constexpr int RW_CENTERS = 192;    // control points one warp stages (even)
 constexpr int RW_CAND = 8;         // candidates one warp stages (more: the unstaged path)
@@ -447,7 +478,7 @@ constexpr int RW_LISTED = 0xffff;  // marks a mini-brick whose cells are evaluat
 struct RasterWarp {
   float4 cw[RW_CENTERS];            // control point pairs at the brick's nearest image
   unsigned char mcls[RW_CAND][64];  // per candidate and mini-brick: class | walker bit << 2
-  uint16_t val[64];                 // per mini-brick: the solid word of all its cells, or RW_LISTED
+  uint16_t val[64];                 // per mini-brick: the word of all its cells, or RW_LISTED
   unsigned char list[64];           // the mini-bricks whose cells are evaluated
   int p[RW_CAND], q0[RW_CAND], q1[RW_CAND], e0[RW_CAND], e1[RW_CAND];
 };
@@ -477,22 +508,26 @@ __device__ __forceinline__ int raster_pieces_log2(uint32_t nlist, uint32_t warps
 //     the candidate with most sub-samples, lowest index on ties.
 // All decisions use bounds with a 1e-3 margin and, within 4e-5 of f = 1, the exact binary32
 // sequence shared with the CPU oracle, so counts and owners equal the oracle's bit for bit.
-// With cells = 0 a launch stops after the masks of step 2: the IBB coupling reads node classes, not
-// counts, and needs only the walkers' masks each step.
+// With nodes the words are the IBB coupling's node classes instead (0, or 1 + the lowest particle
+// holding the cell centre): step 3 then tests one point per cell of the straddling mini-bricks.
+// (A pass of its own over every cell of every brick took 119 us at 256^3, one chain of dependent
+// loads per block; here the candidates are staged and most cells settled, and the raster runs
+// beside the update.)
 struct RasterArgs {
   Geom g;
   ParticleSet ps;
   BrickSet bs;
   uint16_t* solid;
   unsigned long long* status;
-  int cells;
+  uint16_t* nodes;
 };
 
 __device__ __forceinline__ void raster_body(const RasterArgs& A, int blk, int nblk) {
   const Geom g = A.g;
   const ParticleSet ps = A.ps;
   const BrickSet bs = A.bs;
-  uint16_t* __restrict__ solid = A.solid;
+  const bool classes = A.nodes != nullptr;
+  uint16_t* __restrict__ solid = classes ? A.nodes : A.solid;   // the words of cells written
   unsigned long long* __restrict__ status = A.status;
   __shared__ RasterWarp s_rw[RW_WARPS];
   const unsigned full = 0xffffffffu;
@@ -501,8 +536,8 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A, int blk, int nb
   const uint32_t nbrick = (uint32_t)g.nb[0] * g.nb[1] * g.nb[2];
   const uint32_t nlist = bs.bword[nbrick];
   const uint32_t warps = (uint32_t)nblk * RW_WARPS;
-  // the masks alone are two rounds of bounds per brick: whole bricks there
-  const int plog = A.cells ? raster_pieces_log2(nlist, warps) : 0, slog = min(plog, 3), parts = 1 << (plog - slog);
+  // node classes are a few rounds per brick: whole bricks there
+  const int plog = classes ? 0 : raster_pieces_log2(nlist, warps), slog = min(plog, 3), parts = 1 << (plog - slog);
   const uint32_t units = nlist << plog;
   const int K = 64 >> slog;          // mini-bricks per slice: 64, 32, 16 or 8
   const int rows_y = K >= 16 ? 8 : 4;   // cell rows of a slice along y
@@ -602,7 +637,9 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A, int blk, int nb
           }
           listed = listed && bi * BRICK + 2 * (mb & 3) < g.n[0] && bj * BRICK + 2 * ((mb >> 2) & 3) < g.n[1] &&
                    bk * BRICK + 2 * (mb >> 4) < g.n[2];
-          W.val[mb] = listed ? (uint16_t)RW_LISTED : own != 0x7fffffff ? (uint16_t)(64 | (own << 7)) : (uint16_t)0;
+          W.val[mb] = listed ? (uint16_t)RW_LISTED : own == 0x7fffffff ? (uint16_t)0
+                      : classes               ? (uint16_t)(1 + own)
+                                              : (uint16_t)(64 | (own << 7));
         }
         wm[h] = __ballot_sync(full, need);
         const unsigned bl = __ballot_sync(full, listed);
@@ -618,7 +655,7 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A, int blk, int nb
       }
       __syncwarp();
       // cells of the other mini-bricks: two cells of one mini-brick (x, x + 1) per lane
-      if (A.cells && part == 0) {
+      if (part == 0) {
         const int ly0 = 2 * ((mb0 >> 2) & 3), lz0 = 2 * (mb0 >> 4);
         for (int t = lane; t < 4 * K; t += 32) {
           const int r = t >> 2, ly = ly0 + (r & (rows_y - 1)), lz = lz0 + r / rows_y;
@@ -645,7 +682,7 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A, int blk, int nb
     }
     // 3. cells of this part's listed mini-bricks, 32 per round (lane: mini-brick lane / 8, its cell
     // lane & 7)
-    for (int r = part; A.cells && r < nlisted; r += 4 * parts) {
+    for (int r = part; r < nlisted; r += 4 * parts) {
       const int at = r + (lane >> 3) * parts;
       const bool have = at < nlisted;
       const int mb = have ? W.list[at] : 0;
@@ -653,6 +690,25 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A, int blk, int nb
       const int i = bi * BRICK + lx, j = bj * BRICK + ly, k = bk * BRICK + lz;
       const bool in_dom = have && i < g.n[0] && j < g.n[1] && k < g.n[2];
       const float xi = (float)i, yj = (float)j, zk = (float)k;
+      if (classes) {
+        const float xs = xi + 0.5f, ys = yj + 0.5f, zs = zk + 0.5f;
+        int own = 0x7fffffff;
+        for (int m = 0; in_dom && m < (staged ? n : over ? ps.P : (int)nc); ++m) {
+          const int pp = staged ? W.p[m] : over ? m : (bs.bcand[b * MAXC + m] & 0x7fff);
+          if (pp > own) continue;
+          bool in;
+          if (staged) {
+            const int cls = W.mcls[m][mb] & 3;
+            in = cls == 1 || (cls == 2 && (mi ? point_inside<true>(W.cw, W.q0[m], W.q1[m], bs.cworld, W.e0[m], W.e1[m], xs, ys, zs, g)
+                                              : point_inside<false>(W.cw, W.q0[m], W.q1[m], bs.cworld, W.e0[m], W.e1[m], xs, ys, zs, g)));
+          } else {
+            in = inside_exact(bs.cworld, ps.desc[pp].c0, ps.desc[pp].c1, xs, ys, zs, g);
+          }
+          if (in) own = pp;
+        }
+        if (in_dom) solid[((uint32_t)k * g.n[1] + j) * g.n[0] + i] = own == 0x7fffffff ? (uint16_t)0 : (uint16_t)(1 + own);
+        continue;
+      }
       uint64_t any = 0ull;
       int best = 0, bestp = -1;
       unsigned pend = 0u;
@@ -740,14 +796,14 @@ __global__ void __launch_bounds__(256, 4) raster_batched(const RasterArgs* __res
 // one block per SM made the raster itself the longer branch)
 int raster_grid(int nsm) { return nsm * 2; }
 void launch_raster(const Geom& g, const ParticleSet& ps, BrickSet bs, uint16_t* solid,
-                   unsigned long long* status, int nsm, cudaStream_t st, bool cells) {
+                   unsigned long long* status, int nsm, cudaStream_t st, uint16_t* nodes) {
   if (ps.P == 0) return;
-  raster_kernel<<<raster_grid(nsm), RW_WARPS * 32, 0, st>>>(RasterArgs{g, ps, bs, solid, status, cells ? 1 : 0});
+  raster_kernel<<<raster_grid(nsm), RW_WARPS * 32, 0, st>>>(RasterArgs{g, ps, bs, solid, status, nodes});
 }
 size_t raster_args_size() { return sizeof(RasterArgs); }
 void raster_args(void* dst, const Geom& g, const ParticleSet& ps, BrickSet bs, uint16_t* solid,
                  unsigned long long* status) {
-  *static_cast<RasterArgs*>(dst) = RasterArgs{g, ps, bs, solid, status, 1};
+  *static_cast<RasterArgs*>(dst) = RasterArgs{g, ps, bs, solid, status, nullptr};
 }
 void launch_raster_batched(const void* args, const BlockMap* map, int nblocks, cudaStream_t st) {
   if (nblocks > 0) raster_batched<<<nblocks, RW_WARPS * 32, 0, st>>>(static_cast<const RasterArgs*>(args), map);
@@ -853,35 +909,12 @@ void launch_density(int q, int storage, const Geom& g, const void* f, double rho
   RWMI_DISPATCH(q, storage, density_kernel, g, f, rho0, out);
 }
 
-// Is (x, y, z) inside particle [c0, c1) by Eq. 3 in the CPU oracle's binary32 sequence? A fast
-// value (fast reciprocal, contraction allowed; error ~1e-6 relative) decides outside 4e-5 of 1,
-// the exact sequence inside that band, so the answer always equals the exact one.
-__device__ __forceinline__ bool inside_exact(const float4* __restrict__ cw, int c0, int c1, float x, float y,
-                                             float z, const Geom& g) {
-  float f = 0.0f;
-  for (int i = c0; i < c1; ++i) {
-    const float4 c = cw[i];
-    const float dx = min_image_rn(x - c.x, (float)g.n[0], g.wall[0]);
-    const float dy = min_image_rn(y - c.y, (float)g.n[1], g.wall[1]);
-    const float dz = min_image_rn(z - c.z, (float)g.n[2], g.wall[2]);
-    f += __fdividef(c.w, dx * dx + dy * dy + dz * dz);
-  }
-  if (fabsf(f - 1.0f) > 4e-5f) return f >= 1.0f;
-  return metaball_exact(cw, c0, c1, x, y, z, g) >= 1.0f;
-}
-
-// IBB node classes (Section 2.4.3): a cell centre is solid when Eq. 3 of some particle reaches 1
-// there (binary32, the CPU oracle's operation order), owned by the lowest such particle index.
-// Only cells of flagged bricks can be solid. With refill, a node solid in prev and fluid now gets
-// G^eq(rho0, u_new) with u_new its former particle's rigid velocity (Eq. 27).
-// Brick-major: block 2 b + h takes half h (z rows 4 h .. 4 h + 3) of brick b, so that a warp's
-// cells share their brick and its candidate list.
-template <int Q, int STORE>
-__global__ void __launch_bounds__(256) node_kernel(Geom g, ParticleSet ps, BrickSet bs, const uint16_t* __restrict__ prev,
-                                                   uint16_t* __restrict__ cur, void* f_, double rho0_d, int refill) {
-  using L = Lat<Q>;
-  using S = Store<STORE>;
-  using R = typename S::R;
+// IBB node classes (Section 2.4.3) of every cell: a cell centre is solid when Eq. 3 of some particle
+// reaches 1 there (binary32, the CPU oracle's operation order), owned by the lowest such particle
+// index. Only cells of flagged bricks can be solid. Set-up and read-back; in a step the raster
+// writes the classes of flagged bricks and refill_kernel the rest. Brick-major: block 2 b + h takes
+// half h (z rows 4 h .. 4 h + 3) of brick b.
+__global__ void __launch_bounds__(256) node_kernel(Geom g, ParticleSet ps, BrickSet bs, uint16_t* __restrict__ cur) {
   const uint32_t b = blockIdx.x >> 1;
   const uint32_t l = threadIdx.x + ((blockIdx.x & 1u) << 8);
   const uint32_t bi = b % (uint32_t)g.nb[0], bj = (b / (uint32_t)g.nb[0]) % (uint32_t)g.nb[1],
@@ -907,9 +940,39 @@ __global__ void __launch_bounds__(256) node_kernel(Geom g, ParticleSet ps, Brick
     }
   }
   cur[c] = (uint16_t)node;
-  if (refill && node == 0 && prev[c] != 0) {
+}
+
+void launch_nodes(const Geom& g, const ParticleSet& ps, BrickSet bs, uint16_t* cur, cudaStream_t st) {
+  node_kernel<<<2u * (uint32_t)g.nb[0] * (uint32_t)g.nb[1] * (uint32_t)g.nb[2], 256, 0, st>>>(g, ps, bs, cur);
+}
+
+// Ahead of the IBB links of a step: cells of bricks that hold no particle now are fluid (the raster
+// wrote the others), and a node solid in prev and fluid in cur gets G^eq(rho0, u_new) with u_new its
+// former particle's rigid velocity (Eq. 27). One thread per 8 cells of a row (16 bytes of classes)
+// where the rows are aligned, else per cell: a stream over prev and the empty bricks of cur.
+template <int Q, int STORE, int CELLS>
+__global__ void __launch_bounds__(256) refill_kernel(Geom g, BrickSet bs, const uint16_t* __restrict__ prev,
+                                                     uint16_t* __restrict__ cur, void* f_, double rho0_d) {
+  using L = Lat<Q>;
+  using S = Store<STORE>;
+  using R = typename S::R;
+  const uint32_t c0 = (blockIdx.x * blockDim.x + threadIdx.x) * CELLS;
+  if (c0 >= g.ncell) return;
+  const uint32_t z = fast_div(c0, g.mxy, g.sxy), rem = c0 - z * g.nxy, y = fast_div(rem, g.mx, g.sx),
+                 x0 = rem - y * (uint32_t)g.n[0];
+  const bool held = bs.bword[((z >> 3) * (uint32_t)g.nb[1] + (y >> 3)) * (uint32_t)g.nb[0] + (x0 >> 3)] >> 16;
+  if constexpr (CELLS == 8) {
+    const uint4 p8 = *reinterpret_cast<const uint4*>(prev + c0);
+    if (!held) *reinterpret_cast<uint4*>(cur + c0) = make_uint4(0u, 0u, 0u, 0u);
+    if (!(p8.x | p8.y | p8.z | p8.w)) return;
+  } else {
+    if (!held) cur[c0] = 0;
+  }
+  for (uint32_t k = 0; k < CELLS; ++k) {
+    const uint32_t c = c0 + k, was = prev[c];
+    if (was == 0 || cur[c] != 0) continue;
     R un[3];
-    rigid_velocity<R>(g, bs.pose, bs.posed, (int)prev[c] - 1, (R)x + R(0.5), (R)y + R(0.5), (R)z + R(0.5), un);
+    rigid_velocity<R>(g, bs.pose, bs.posed, (int)was - 1, (R)(x0 + k) + R(0.5), (R)y + R(0.5), (R)z + R(0.5), un);
     const R rho0 = (R)rho0_d, uu = un[0] * un[0] + un[1] * un[1] + un[2] * un[2];
     typename S::T* f = (typename S::T*)f_;
 #pragma unroll
@@ -922,21 +985,19 @@ __global__ void __launch_bounds__(256) node_kernel(Geom g, ParticleSet ps, Brick
   }
 }
 
-void launch_nodes(int q, int storage, const Geom& g, const ParticleSet& ps, BrickSet bs,
-                  const uint16_t* prev, uint16_t* cur, void* f, double rho0, bool refill,
-                  cudaStream_t st) {
-  const dim3 grid_(2u * (uint32_t)g.nb[0] * (uint32_t)g.nb[1] * (uint32_t)g.nb[2]);   // two blocks per brick
-  if (q == 15) {
-    if (storage == 0) node_kernel<15, 0><<<grid_, 256, 0, st>>>(g, ps, bs, prev, cur, f, rho0, refill ? 1 : 0);
-    else if (storage == 1) node_kernel<15, 1><<<grid_, 256, 0, st>>>(g, ps, bs, prev, cur, f, rho0, refill ? 1 : 0);
-    else if (storage == 2) node_kernel<15, 2><<<grid_, 256, 0, st>>>(g, ps, bs, prev, cur, f, rho0, refill ? 1 : 0);
-    else node_kernel<15, 3><<<grid_, 256, 0, st>>>(g, ps, bs, prev, cur, f, rho0, refill ? 1 : 0);
-  } else {
-    if (storage == 0) node_kernel<19, 0><<<grid_, 256, 0, st>>>(g, ps, bs, prev, cur, f, rho0, refill ? 1 : 0);
-    else if (storage == 1) node_kernel<19, 1><<<grid_, 256, 0, st>>>(g, ps, bs, prev, cur, f, rho0, refill ? 1 : 0);
-    else if (storage == 2) node_kernel<19, 2><<<grid_, 256, 0, st>>>(g, ps, bs, prev, cur, f, rho0, refill ? 1 : 0);
-    else node_kernel<19, 3><<<grid_, 256, 0, st>>>(g, ps, bs, prev, cur, f, rho0, refill ? 1 : 0);
-  }
+void launch_refill(int q, int storage, const Geom& g, BrickSet bs, const uint16_t* prev, uint16_t* cur, void* f,
+                   double rho0, cudaStream_t st) {
+  const bool rows = g.n[0] % 8 == 0;   // every row then starts on a 16-byte boundary
+  const uint32_t threads = rows ? g.ncell / 8 : g.ncell, blocks = (threads + 255) / 256;
+#define RWMI_REFILL(QQ, SS)                                                                              \
+  do {                                                                                                 \
+    if (rows) refill_kernel<QQ, SS, 8><<<blocks, 256, 0, st>>>(g, bs, prev, cur, f, rho0);               \
+    else refill_kernel<QQ, SS, 1><<<blocks, 256, 0, st>>>(g, bs, prev, cur, f, rho0);                    \
+  } while (0)
+  // IBB is built for binary32-shifted and binary64 storage
+  if (q == 15) { if (storage == 3) RWMI_REFILL(15, 3); else RWMI_REFILL(15, 1); }
+  else { if (storage == 3) RWMI_REFILL(19, 3); else RWMI_REFILL(19, 1); }
+#undef RWMI_REFILL
 }
 
 __global__ void unpack_solid_kernel(Geom g, const uint16_t* solid, const uint32_t* bword,

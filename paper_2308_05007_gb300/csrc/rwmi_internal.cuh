@@ -251,9 +251,10 @@ void launch_force_row(const double* acc, int P, double* base, int interval, int 
 void launch_pose_bin(const Geom& g, const ParticleSet& ps, BrickSet bs, const int64_t* d_T,
                      int t_offset, const double F0[3], double force_period, int zero_forces,
                      double* forces, int q, double tau, cudaStream_t st);
-// cells = false: brick classes and walker masks only (no per-cell sub-sample counts)
+// sub-sample counts and owners into solid, or, with nodes, the IBB node classes of the bricks that
+// hold a particle into nodes; and the walkers' masks
 void launch_raster(const Geom& g, const ParticleSet& ps, BrickSet bs, uint16_t* solid,
-                   unsigned long long* status, int nsm, cudaStream_t st, bool cells = true);
+                   unsigned long long* status, int nsm, cudaStream_t st, uint16_t* nodes = nullptr);
 // Extra inputs of the IBB coupling: node classes of this time, (u, rho) of the previous update,
 // particle descriptors (control point ranges). nullptr selects the partially saturated cells.
 struct IbbArgs {
@@ -261,13 +262,14 @@ struct IbbArgs {
   const float4* uprev = nullptr;
   const ParticleDesc* desc = nullptr;
   const int32_t* base = nullptr;   // per cell: index of its first link in q (ibb links)
-  const uint32_t* word = nullptr;  // per cell of a flagged brick: bit 0 solid node, bit i link i
+  const uint32_t* word = nullptr;  // per cell of a masked mini-brick: bit 0 solid node, bit i link i
+  const uint64_t* mask = nullptr;  // per brick: the mini-bricks that may hold solid nodes or links
   const float* q = nullptr;        // q of every link (Eq. 25)
   const void* g = nullptr;         // G_i of every link (Eqs. 23-25), in the arithmetic type
   int cap = 0;                     // capacity of the link list
 };
 // The IBB link list of a context: per cell the index of its first link (or -1 - its overflow
-// slot) and its node word; per link the cell, the direction | particle << 8, q and G_i (binary32
+// slot) and its node word; per link the cell, the direction, q and G_i (binary32
 // or binary64, 8 bytes reserved). q and G hold cap list entries followed by ocap overflow slots of
 // Q - 1 links each (cells whose links did not fit in the list; ocell lists them). count: list and
 // overflow append counters, two time parities each.
@@ -341,11 +343,12 @@ void launch_dem_init(const DemArgs& a, cudaStream_t st);
 // body frames (cbody) and the state origins to the centres of mass
 void launch_dem_mass(const DemArgs& a, unsigned long long* sums, const double* density, double* mass, double* Ib,
                      double* props, float4* cbody, cudaStream_t st);
-// IBB node classes at time t (bricks bs of that time) into cur; with refill, nodes solid in prev
-// and fluid now get the equilibrium at their former particle's rigid velocity (Eq. 27).
-void launch_nodes(int q, int storage, const Geom& g, const ParticleSet& ps, BrickSet bs,
-                  const uint16_t* prev, uint16_t* cur, void* f, double rho0, bool refill,
-                  cudaStream_t st);
+// IBB node classes of all cells at the time of bricks bs into cur (set-up, read-back)
+void launch_nodes(const Geom& g, const ParticleSet& ps, BrickSet bs, uint16_t* cur, cudaStream_t st);
+// Completes the raster's classes cur of this time (0 in bricks without a particle); nodes solid in
+// prev and fluid now get the equilibrium at their former particle's rigid velocity (Eq. 27).
+void launch_refill(int q, int storage, const Geom& g, BrickSet bs, const uint16_t* prev, uint16_t* cur, void* f,
+                   double rho0, cudaStream_t st);
 void launch_init_populations(int q, int storage, const Geom& g, void* f, double rho0,
                              const double u0[3], float* u, cudaStream_t st);
 // Time of a launch: *d_T (the step counter at the start of the current run of steps, advanced

@@ -41,6 +41,21 @@ template <int Q> struct Lat {
   }
 };
 
+// Components and weight of a direction known only at run time: two bits per direction in one
+// 64-bit constant per axis (evaluating Lat's constant expressions there took chains of selects).
+template <int Q> __host__ __device__ constexpr uint64_t packed_axis(int a) {
+  uint64_t v = 0;
+  for (int i = 0; i < Q; ++i) v |= (uint64_t)(Lat<Q>::e(i, a) + 1) << (2 * i);
+  return v;
+}
+template <int Q, int A> __device__ __forceinline__ int dir_e(int i) {
+  constexpr uint64_t t = packed_axis<Q>(A);
+  return (int)((t >> (2 * i)) & 3u) - 1;
+}
+template <int Q, typename R> __device__ __forceinline__ R dir_wt(int i) {   // i >= 1
+  const int e2 = (dir_e<Q, 0>(i) & 1) + (dir_e<Q, 1>(i) & 1) + (dir_e<Q, 2>(i) & 1);
+  return e2 == 1 ? Lat<Q>::template wt<R>(1) : Lat<Q>::template wt<R>(4);
+}
 
 // Population storage: binary32 f_i, binary32 f_i - w_i rho0 ("shifted"), binary16 shifted (all
 // with binary32 arithmetic), or binary64 shifted with binary64 arithmetic.

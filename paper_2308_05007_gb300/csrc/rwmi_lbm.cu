@@ -86,8 +86,7 @@ template <int STORE> struct TmaRow {
 // wrap); false where x - e_d lies beyond a plane wall.
 template <int Q, bool WALLS>
 __device__ __forceinline__ bool pull_source(const Geom& g, uint32_t x, uint32_t y, uint32_t z, int d, int& off) {
-  using L = Lat<Q>;
-  const int ex = L::e(d, 0), ey = L::e(d, 1), ez = L::e(d, 2);
+  const int ex = dir_e<Q, 0>(d), ey = dir_e<Q, 1>(d), ez = dir_e<Q, 2>(d);
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const int sy = nx, sz = (int)g.nxy;
   if (WALLS && ((g.wall[0] && ((ex > 0 && x == 0) || (ex < 0 && (int)x == nx - 1))) ||
@@ -116,7 +115,7 @@ ibb_link_value(const Geom& g, const typename Store<STORE>::T* __restrict__ in0, 
   using S = Store<STORE>;
   using R = typename S::R;
   const int ip = L::opp(i);
-  const int ex = L::e(ip, 0), ey = L::e(ip, 1), ez = L::e(ip, 2);   // into the wall
+  const int ex = dir_e<Q, 0>(ip), ey = dir_e<Q, 1>(ip), ez = dir_e<Q, 2>(ip);   // into the wall
   xw[0] = (R)x + R(0.5) + qf * (R)ex;
   xw[1] = (R)y + R(0.5) + qf * (R)ey;
   xw[2] = (R)z + R(0.5) + qf * (R)ez;
@@ -137,7 +136,7 @@ ibb_link_value(const Geom& g, const typename Store<STORE>::T* __restrict__ in0, 
     const R us2 = (R(1) - qf) / (R(1) + qf) * uff[a] + R(2) * qf / (R(1) + qf) * uw[a];
     ud[a] = us1 / R(3) + R(2) * us2 / R(3);
   }
-  const R w = L::template wt<R>(ip);
+  const R w = dir_wt<Q, R>(ip);
   const R eud = (R)ex * ud[0] + (R)ey * ud[1] + (R)ez * ud[2];
   const R euf = (R)ex * uf[0] + (R)ey * uf[1] + (R)ez * uf[2];
   const R uud = ud[0] * ud[0] + ud[1] * ud[1] + ud[2] * ud[2];
@@ -161,8 +160,8 @@ __device__ __forceinline__ void ibb_link_force(const Geom& g, const PoseF* __res
   using S = Store<STORE>;
   using R = typename S::R;
   const int ip = L::opp(i);
-  const R ex = (R)L::e(ip, 0), ey = (R)L::e(ip, 1), ez = (R)L::e(ip, 2);
-  const R w = L::template wt<R>(ip);
+  const R ex = (R)dir_e<Q, 0>(ip), ey = (R)dir_e<Q, 1>(ip), ez = (R)dir_e<Q, 2>(ip);
+  const R w = dir_wt<Q, R>(ip);
   const R sh = S::shifted ? w * rho0 : R(0);
   const R gp = Gp + sh, gi = G + sh;
   Fl[0] = (ex - uw[0]) * gp - (-ex - uw[0]) * gi;
@@ -209,7 +208,7 @@ __device__ __forceinline__ void ibb_cell_force(const Geom& g, const typename Sto
     const int p = (int)nodes[c + off] - 1;
     const R qf = (R)ib_q[kk];
     const R G = ib_g[kk];
-    const int ex = L::e(ip, 0), ey = L::e(ip, 1), ez = L::e(ip, 2);
+    const int ex = dir_e<Q, 0>(ip), ey = dir_e<Q, 1>(ip), ez = dir_e<Q, 2>(ip);
     const R xw[3] = {(R)x + R(0.5) + qf * (R)ex, (R)y + R(0.5) + qf * (R)ey, (R)z + R(0.5) + qf * (R)ez};
     R uw[3];
     rigid_velocity<R>(g, pose, posed, p, xw[0], xw[1], xw[2], uw);
@@ -260,7 +259,7 @@ __device__ __forceinline__ void lbm_body(Geom g, Planes<Q, typename Store<STORE>
                                                   const uint32_t* __restrict__ ib_word,
                                                   const float* __restrict__ ib_q,
                                                   const typename Store<STORE>::R* __restrict__ ib_g, int ib_cap,
-                                                  int blk, const typename Store<STORE>::T* srow = nullptr,
+                                                  const uint64_t* __restrict__ ib_mask, int blk, const typename Store<STORE>::T* srow = nullptr,
                                                   uint32_t staged_idx = 0, bool staged_valid = false,
                                                   int staged_lx = 0) {
   using L = Lat<Q>;
@@ -331,13 +330,13 @@ __device__ __forceinline__ void lbm_body(Geom g, Planes<Q, typename Store<STORE>
   R Fib[3] = {R(0), R(0), R(0)}, Tib[3] = {R(0), R(0), R(0)};   // IBB: this cell's link forces
   int ib_owner = -1;
   if constexpr (IBB) {
-    // ibb_links_kernel, which ran before, left every cell of a flagged brick its node word: bit 0
-    // a solid node, bit i a link (x - e_i a solid node, not beyond a wall), and ibb_link_kernel
-    // left q and G_i of every link. Cells of other bricks have no solid neighbour (the IBB brick
-    // radius is at least rb + sqrt 3).
+    // ibb_links_kernel, which ran before, left every cell of a masked mini-brick of a flagged brick
+    // its node word: bit 0 a solid node, bit i a link (x - e_i a solid node, not beyond a wall), and
+    // ibb_link_kernel left q and G_i of every link. Other cells have no solid neighbour (the IBB
+    // brick radius is at least rb + sqrt 3, the mask's reach sqrt(3) + 1.75 from the mini-brick's centre).
     unsigned lmask = 0u;
     const uint32_t bq = ((z >> 3) * (uint32_t)g.nb[1] + (y >> 3)) * (uint32_t)g.nb[0] + (x >> 3);
-    if (valid && (bword[bq] >> 16)) {
+    if (valid && (bword[bq] >> 16) && ((ib_mask[bq] >> (((x >> 1) & 3u) + 2u * (y & 6u) + 8u * (z & 6u))) & 1ull)) {
       const uint32_t lw = ib_word[c];
       solid_self = (lw & 1u) != 0u;
       lmask = lw & ~1u;
@@ -691,9 +690,9 @@ lbm_kernel(Geom g, Planes<Q, typename Store<STORE>::T> pl, float4* __restrict__ 
            double* __restrict__ forces, const uint16_t* __restrict__ nodes, const float4* __restrict__ uprev,
            const ParticleDesc* __restrict__ desc, const float4* __restrict__ cworld,
            const int32_t* __restrict__ ib_base, const uint32_t* __restrict__ ib_word, const float* __restrict__ ib_q,
-           const typename Store<STORE>::R* __restrict__ ib_g, int ib_cap) {
+           const typename Store<STORE>::R* __restrict__ ib_g, int ib_cap, const uint64_t* __restrict__ ib_mask) {
   lbm_body<Q, STORE, WALLS, MODE, IBB>(g, pl, u4, solid, bword, pose, posed, sp, tau, omega, guo0, rho0, red, forces,
-                                       nodes, uprev, desc, cworld, ib_base, ib_word, ib_q, ib_g, ib_cap, blockIdx.x);
+                                       nodes, uprev, desc, cworld, ib_base, ib_word, ib_q, ib_g, ib_cap, ib_mask, blockIdx.x);
   // launched behind the raster (launch_lbm's after_raster): one block outlasts it, so that whatever
   // follows this kernel on the stream follows the raster too (returns at once otherwise)
   if (blockIdx.x == gridDim.x - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -708,37 +707,27 @@ __global__ void __launch_bounds__(256, sizeof(typename Store<STORE>::R) == 8 ? 2
   const LbmArgs<Q, STORE>& a = args[m.domain];
   lbm_body<Q, STORE, WALLS, MODE, IBB>(a.g, a.pl, a.u4, a.solid, a.bword, a.pose, a.posed, a.sp, a.tau, a.omega,
                                        a.guo0, a.rho0, a.red, a.forces, nullptr, nullptr, nullptr, nullptr,
-                                       nullptr, nullptr, nullptr, nullptr, 0, m.block);
+                                       nullptr, nullptr, nullptr, nullptr, 0, nullptr, m.block);
 }
 #undef RWMI_LBM_BOUNDS
 
 // ---- IBB links (Eq. 25) ahead of the LBM update ------------------------------------------
 // Every fluid node of a flagged brick whose lattice neighbour x - e_i is a solid node owns the
-// link (x, i). ibb_links_kernel gives every cell of a flagged brick its node word (bit 0: solid
+// link (x, i). ibb_links_kernel gives every cell of a masked mini-brick its node word (bit 0: solid
 // node; bit i: link i), appends a node's links in direction order (warp-aggregated) and keeps the
 // index of its first one (or, when the list is full, an overflow slot); ibb_link_kernel then runs
 // the 24-step binary32 bisection of every link and forms its G at full occupancy, instead of
-// inside the update.
+// inside the update. A warp takes a quarter of a flagged brick of the raster's list, leaves it at once
+// when no mini-brick of it has the walkers' mask bit (most have none), and reserves list entries
+// once for its 128 cells. (A reservation per 32 cells, all on one counter, bound this pass: 105 us at
+// 256^3 with a block per half brick of the whole box, 77 us with a warp per 32 cells; a whole brick
+// per warp took 115 us, its rows waiting for one another.)
+constexpr int LINK_WARPS = 8, LINK_ROWS = 4;
+// Node word of cell c = (x, y, z): bit 0 a solid node, bit i a link (x - e_i solid, not beyond a wall).
 template <int Q, bool WALLS>
-__global__ void __launch_bounds__(256) ibb_links_kernel(Geom g, const uint32_t* __restrict__ bword,
-                                                        const uint16_t* __restrict__ nodes,
-                                                        int32_t* __restrict__ base, uint32_t* __restrict__ word,
-                                                        uint32_t* __restrict__ lcell,
-                                                        uint32_t* __restrict__ lmeta, unsigned int* count, int cap,
-                                                        int32_t* __restrict__ ocell, unsigned int* ocount, int ocap,
-                                                        unsigned long long* __restrict__ status) {
+__device__ __forceinline__ unsigned node_word(const Geom& g, const uint16_t* __restrict__ nodes, int c, uint32_t x,
+                                              uint32_t y, uint32_t z) {
   using L = Lat<Q>;
-  // brick-major (as node_kernel): block 2 b + h takes half h of brick b; bricks that hold no
-  // particle have no links and leave at once
-  const uint32_t bq = blockIdx.x >> 1;
-  if (!(bword[bq] >> 16)) return;   // block-uniform
-  const uint32_t l = threadIdx.x + ((blockIdx.x & 1u) << 8);
-  const uint32_t bi = bq % (uint32_t)g.nb[0], bj = (bq / (uint32_t)g.nb[0]) % (uint32_t)g.nb[1],
-                 bk = bq / ((uint32_t)g.nb[0] * (uint32_t)g.nb[1]);
-  uint32_t x = bi * BRICK + (l & 7u), y = bj * BRICK + ((l >> 3) & 7u), z = bk * BRICK + (l >> 6);
-  const bool valid = x < (uint32_t)g.n[0] && y < (uint32_t)g.n[1] && z < (uint32_t)g.n[2];
-  if (!valid) { x = 0; y = 0; z = 0; }   // outside the box (partial brick): no links
-  const int c = (int)((z * (uint32_t)g.n[1] + y) * (uint32_t)g.n[0] + x);
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const int sy = nx, sz = (int)g.nxy;
   const int ox_p = x == 0 ? nx - 1 : -1, ox_m = (int)x == nx - 1 ? -(nx - 1) : 1;
@@ -747,60 +736,92 @@ __global__ void __launch_bounds__(256) ibb_links_kernel(Geom g, const uint32_t* 
   const bool wx_p = WALLS && g.wall[0] && x == 0, wx_m = WALLS && g.wall[0] && (int)x == nx - 1;
   const bool wy_p = WALLS && g.wall[1] && y == 0, wy_m = WALLS && g.wall[1] && (int)y == ny - 1;
   const bool wz_p = WALLS && g.wall[2] && z == 0, wz_m = WALLS && g.wall[2] && (int)z == nz - 1;
-  auto off_of = [&](int i) {
-    const int ex = L::e(i, 0), ey = L::e(i, 1), ez = L::e(i, 2);
-    return (ex > 0 ? ox_p : ex < 0 ? ox_m : 0) + (ey > 0 ? oy_p : ey < 0 ? oy_m : 0) +
-           (ez > 0 ? oz_p : ez < 0 ? oz_m : 0);
-  };
-  auto blocked = [&](int i) {
-    const int ex = L::e(i, 0), ey = L::e(i, 1), ez = L::e(i, 2);
-    return (ex > 0 && wx_p) || (ex < 0 && wx_m) || (ey > 0 && wy_p) || (ey < 0 && wy_m) ||
-           (ez > 0 && wz_p) || (ez < 0 && wz_m);
-  };
-  unsigned lmask = 0u;
-  if (valid) {
-    const bool solid_node = nodes[c] != 0;
-    if (!solid_node) {
+  if (nodes[c] != 0) return 1u;
+  unsigned word = 0u;
 #pragma unroll
-      for (int i = 1; i < Q; ++i)
-        if (!blocked(i) && nodes[c + off_of(i)] != 0) lmask |= 1u << i;
-    }
-    word[c] = lmask | (solid_node ? 1u : 0u);
+  for (int i = 1; i < Q; ++i) {
+    const int ex = L::e(i, 0), ey = L::e(i, 1), ez = L::e(i, 2);
+    const bool blocked = (ex > 0 && wx_p) || (ex < 0 && wx_m) || (ey > 0 && wy_p) || (ey < 0 && wy_m) ||
+                         (ez > 0 && wz_p) || (ez < 0 && wz_m);
+    const int off = (ex > 0 ? ox_p : ex < 0 ? ox_m : 0) + (ey > 0 ? oy_p : ey < 0 ? oy_m : 0) +
+                    (ez > 0 ? oz_p : ez < 0 ? oz_m : 0);
+    if (!blocked && nodes[c + off] != 0) word |= 1u << i;
   }
+  return word;
+}
+
+template <int Q, bool WALLS>
+__global__ void __launch_bounds__(LINK_WARPS * 32)
+ibb_links_kernel(Geom g, const uint32_t* __restrict__ bword, const int32_t* __restrict__ rlist,
+                 const uint64_t* __restrict__ wmask, const uint16_t* __restrict__ nodes, int32_t* __restrict__ base,
+                 uint32_t* __restrict__ word, uint32_t* __restrict__ lcell, uint32_t* __restrict__ lmeta,
+                 unsigned int* count, int cap, int32_t* __restrict__ ocell, unsigned int* ocount, int ocap,
+                 unsigned long long* __restrict__ status) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int nl = __popc(lmask);
-  int incl = nl;
+  // a unit: the four rows of four mini-bricks (x 0-7, two y, two z: 32 cells each) at one z of a brick
+  const uint32_t units = bword[(uint32_t)g.nb[0] * g.nb[1] * g.nb[2]] << 2;
+  for (uint32_t u = blockIdx.x * LINK_WARPS + (threadIdx.x >> 5); u < units; u += gridDim.x * LINK_WARPS) {
+    const uint32_t b = (uint32_t)rlist[u >> 2], zq = u & 3u;
+    const uint32_t need = (uint32_t)(wmask[b] >> (16u * zq)) & 0xffffu;
+    if (!need) continue;   // warp-uniform
+    const uint32_t bi = b % (uint32_t)g.nb[0], bj = (b / (uint32_t)g.nb[0]) % (uint32_t)g.nb[1],
+                   bk = b / ((uint32_t)g.nb[0] * (uint32_t)g.nb[1]);
+    const uint32_t x = bi * BRICK + (lane & 7), z = bk * BRICK + 2u * zq + (lane >> 4);
+    unsigned links[LINK_ROWS];
+    int nl = 0;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(full, incl, o);
-    if (lane >= o) incl += v;
-  }
-  const int total = __shfl_sync(full, incl, 31);
-  if (total == 0) return;   // warp-uniform
-  unsigned first = 0;
-  if (lane == 31) first = atomicAdd(count, (unsigned)total);
-  first = __shfl_sync(full, first, 31) + (unsigned)(incl - nl);
-  if (!nl) return;
-  if (first + (unsigned)nl > (unsigned)cap) {   // the list is full: the cell takes an overflow slot
-    for (unsigned k = first; k < (unsigned)cap && k < first + (unsigned)nl; ++k)
-      lcell[k] = 0xffffffffu;   // its reserved list entries stay empty (ibb_link_kernel skips them)
-    const unsigned slot = atomicAdd(ocount, 1u);
-    if (slot < (unsigned)ocap) {
-      ocell[slot] = c;
-      base[c] = -1 - (int32_t)slot;
-    } else {   // both full: this step's result is incomplete (rwmi_sync reports it)
-      atomicAdd(&status[ST_IBB_OVERFLOW], 1ull);
-      word[c] = 0u;   // the cell keeps its pulled populations
+    for (int r = 0; r < LINK_ROWS; ++r) {
+      const uint32_t y = bj * BRICK + 2u * r + ((lane >> 3) & 1);
+      links[r] = 0u;
+      if (((need >> (4 * r + ((lane & 7) >> 1))) & 1u) && x < (uint32_t)g.n[0] && y < (uint32_t)g.n[1] &&
+          z < (uint32_t)g.n[2]) {
+        const int c = (int)((z * (uint32_t)g.n[1] + y) * (uint32_t)g.n[0] + x);
+        const unsigned w = node_word<Q, WALLS>(g, nodes, c, x, y, z);
+        word[c] = w;
+        links[r] = w & ~1u;
+      }
+      nl += __popc(links[r]);
     }
-    return;
-  }
-  base[c] = (int32_t)first;
-  unsigned k = first;
-  for (unsigned m = lmask; m; m &= m - 1u, ++k) {
-    const int i = __ffs(m) - 1;
-    lcell[k] = (uint32_t)c;
-    lmeta[k] = (uint32_t)i | ((uint32_t)(nodes[c + off_of(i)] - 1) << 8);
+    int incl = nl;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(full, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const int total = __shfl_sync(full, incl, 31);
+    if (total == 0) continue;   // warp-uniform
+    unsigned first = 0;
+    if (lane == 31) first = atomicAdd(count, (unsigned)total);
+    first = __shfl_sync(full, first, 31) + (unsigned)(incl - nl);
+#pragma unroll
+    for (int r = 0; r < LINK_ROWS; ++r) {
+      const unsigned n = (unsigned)__popc(links[r]);
+      if (!n) continue;
+      const uint32_t y = bj * BRICK + 2u * r + ((lane >> 3) & 1);
+      const int c = (int)((z * (uint32_t)g.n[1] + y) * (uint32_t)g.n[0] + x);
+      if (first + n > (unsigned)cap) {   // the list is full: the cell takes an overflow slot
+        for (unsigned k = first; k < (unsigned)cap && k < first + n; ++k)
+          lcell[k] = 0xffffffffu;   // its reserved list entries stay empty (ibb_link_kernel skips them)
+        const unsigned slot = atomicAdd(ocount, 1u);
+        if (slot < (unsigned)ocap) {
+          ocell[slot] = c;
+          base[c] = -1 - (int32_t)slot;
+        } else {   // both full: this step's result is incomplete (rwmi_sync reports it)
+          atomicAdd(&status[ST_IBB_OVERFLOW], 1ull);
+          word[c] = 0u;   // the cell keeps its pulled populations
+        }
+      } else {
+        base[c] = (int32_t)first;
+        unsigned k = first;
+        for (unsigned m = links[r]; m; m &= m - 1u, ++k) {
+          lcell[k] = (uint32_t)c;
+          lmeta[k] = (uint32_t)(__ffs(m) - 1);
+        }
+      }
+      first += n;
+    }
+    __syncwarp();
   }
 }
 
@@ -833,12 +854,14 @@ __global__ void __launch_bounds__(256) ibb_link_kernel(Geom g, const float4* __r
   for (unsigned j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
     if (lcell[j] == 0xffffffffu) continue;   // reserved by a cell that went to the overflow slots
     const int c = (int)lcell[j];
-    const uint32_t meta = lmeta[j];
     const uint32_t z = fast_div((uint32_t)c, g.mxy, g.sxy), r = (uint32_t)c - z * g.nxy;
     const uint32_t y = fast_div(r, g.mx, g.sx), x = r - y * g.n[0];
-    const int i = (int)(meta & 31u), p = (int)(meta >> 8), ip = L::opp(i);
+    const int i = (int)lmeta[j], ip = L::opp(i);
+    int off = 0;
+    pull_source<Q, WALLS>(g, x, y, z, i, off);   // a link's source is never beyond a wall
+    const int p = (int)nodes[c + off] - 1;
     const float qv = ibb_link_q(cworld, desc[p].c0, desc[p].c1, (float)x + 0.5f, (float)y + 0.5f, (float)z + 0.5f,
-                                L::e(ip, 0), L::e(ip, 1), L::e(ip, 2), g);
+                                dir_e<Q, 0>(ip), dir_e<Q, 1>(ip), dir_e<Q, 2>(ip), g);
     qout[j] = qv;
     R sum = R(0);   // rho_f: x_f's own post-collision populations, summed in direction order
 #pragma unroll
@@ -868,7 +891,7 @@ __global__ void __launch_bounds__(256) ibb_link_kernel(Geom g, const float4* __r
       pull_source<Q, WALLS>(g, x, y, z, i, off);
       const int p = (int)nodes[c + off] - 1;
       const float qv = ibb_link_q(cworld, desc[p].c0, desc[p].c1, (float)x + 0.5f, (float)y + 0.5f, (float)z + 0.5f,
-                                  L::e(ip, 0), L::e(ip, 1), L::e(ip, 2), g);
+                                  dir_e<Q, 0>(ip), dir_e<Q, 1>(ip), dir_e<Q, 2>(ip), g);
       const size_t kk = (size_t)cap + (size_t)s * (Q - 1) + (size_t)(i - 1);
       qout[kk] = qv;
       R Gp, xw[3], uw[3];
@@ -882,7 +905,6 @@ void launch_ibb_links(int q, int storage, const Geom& g, BrickSet bs, const uint
                       int par, const ParticleDesc* desc, const void* fin, const float* uprev, double rho0,
                       unsigned long long* status, int nsm, cudaStream_t st) {
   const bool walls = g.wall[0] || g.wall[1] || g.wall[2];
-  const unsigned blocks = 2u * (unsigned)g.nb[0] * (unsigned)g.nb[1] * (unsigned)g.nb[2];   // two per brick
   unsigned int* cnt = lk.count + (par & 1);
   unsigned int* nxt = lk.count + ((par + 1) & 1);
   unsigned int* ocnt = lk.count + 2 + (par & 1);
@@ -892,9 +914,10 @@ void launch_ibb_links(int q, int storage, const Geom& g, BrickSet bs, const uint
   do {                                                                                                             \
     using T_ = typename Store<SS>::T;                                                                              \
     using R_ = typename Store<SS>::R;                                                                              \
-    ibb_links_kernel<QQ, WW><<<blocks, 256, 0, st>>>(g, bs.bword, nodes, lk.base, lk.word, lk.cell, lk.meta, cnt,   \
-                                                      lk.cap, lk.ocell, ocnt, lk.ocap, status);                    \
-    ibb_link_kernel<QQ, SS, WW><<<nsm * 8, 256, 0, st>>>(g, bs.cworld, desc, lk.cell, lk.meta, cnt, nxt, lk.cap,   \
+    ibb_links_kernel<QQ, WW><<<nsm * 8, LINK_WARPS * 32, 0, st>>>(g, bs.bword, bs.rlist, bs.wmask, nodes, lk.base, \
+                                                                  lk.word, lk.cell, lk.meta, cnt, lk.cap, lk.ocell, \
+                                                                  ocnt, lk.ocap, status);                           \
+    ibb_link_kernel<QQ, SS, WW><<<nsm * 16, 256, 0, st>>>(g, bs.cworld, desc, lk.cell, lk.meta, cnt, nxt, lk.cap,   \
                                                          lk.q, static_cast<R_*>(lk.g), static_cast<const T_*>(fin),\
                                                          u4, nodes, bs.pose, bs.posed, (R_)rho0, lk.word,          \
                                                          lk.ocell, ocnt, onxt, lk.ocap);                           \
@@ -941,7 +964,7 @@ static void launch_lbm_q(bool walls, bool reduce, const Geom& g, const void* fin
   }
   const int bsz_ok = (bsz == 64 || bsz == 128) ? bsz : 256;
   const dim3 grid((g.ncell + bsz_ok - 1) / bsz_ok), block(bsz_ok);
-#define RWMI_LBM_ARGS g, pl, reinterpret_cast<float4*>(u), solid, bs.bword, bs.pose, bs.posed, bs.sp, (R)tau, (R)(1.0 / tau), (R)(1.0 - 0.5 / tau), (R)rho0, red, forces, ib.nodes, ib.uprev, ib.desc, bs.cworld, ib.base, ib.word, ib.q, static_cast<const R*>(ib.g), ib.cap
+#define RWMI_LBM_ARGS g, pl, reinterpret_cast<float4*>(u), solid, bs.bword, bs.pose, bs.posed, bs.sp, (R)tau, (R)(1.0 / tau), (R)(1.0 - 0.5 / tau), (R)rho0, red, forces, ib.nodes, ib.uprev, ib.desc, bs.cworld, ib.base, ib.word, ib.q, static_cast<const R*>(ib.g), ib.cap, ib.mask
   if constexpr (STORE == 1 || STORE == 3) {   // the fused mode of free-DEM runs
     if (fused) {
       if (walls) launch_kernel(lbm_kernel<Q, STORE, true, 2, IBB>, grid, block, st, after_raster, RWMI_LBM_ARGS);
@@ -1111,7 +1134,7 @@ lbm_tma_kernel(const __grid_constant__ CUtensorMap tin, Geom g, Planes<Q, typena
     const uint32_t c = (uint32_t)row * (uint32_t)nx + (uint32_t)(x0 + lx);
     lbm_body<Q, STORE, WALLS, 0, false, true>(g, pl, u4, solid, bword, pose, posed, sp, tau, omega, guo0, rho0,
                                               nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-                                              nullptr, nullptr, 0, 0, stage, c, valid, lx);
+                                              nullptr, nullptr, 0, nullptr, 0, stage, c, valid, lx);
     __syncthreads();   // every lane is done with this buffer
     if (tid == 0) {
       const int tn = t + TMA_STAGES * gridDim.x;

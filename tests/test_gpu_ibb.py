@@ -186,3 +186,56 @@ def test_ibb_overlapping_pair_force_is_galilean_invariant(storage, tol):
     print(f"IBB storage {storage}: |F_x(U) - F_x(0)| = {np.abs(fm[:, 0] - fr[:, 0]).max():.2e}")
     assert fr[0, 0] > 15.0 and fr[1, 0] < -15.0
     np.testing.assert_allclose(fm[:, 0], fr[:, 0], rtol=0, atol=tol)
+
+
+def _shapes(name):
+    """dims, walls and particles [(origin, centres, sigma, k range)] of a link test."""
+    return {
+        "one_centre": ((26, 24, 22), 4, [((13.2, 11.7, 11.1), 1, 0.0, (30.0, 30.0))]),
+        "small_weights": ((24, 26, 28), 0, [((9.3, 12.2, 14.4), 5, 1.0, (0.4, 0.9)), ((18.4, 17.1, 8.2), 2, 0.6, (1.0, 2.0))]),
+        "across_faces": ((22, 21, 20), 0, [((0.4, 20.6, 0.2), 4, 1.2, (3.0, 6.0))]),       # rows of 22 cells: refilled cell by cell
+        "box_of_a_particle": ((15, 14, 16), 0, [((7.0, 7.0, 8.0), 3, 1.0, (4.0, 6.0))]),   # points near half the box
+        "many_centres": ((44, 40, 36), 4, [((22.0, 20.0, 18.0), 40, 4.0, (0.5, 1.5))]),    # uneven surface, grazing links
+        "long_box": ((600, 18, 16), 0, [((590.3, 9.2, 8.1), 3, 1.0, (4.0, 6.0)), ((300.6, 8.8, 7.9), 2, 1.0, (6.0, 9.0))]),
+    }[name]
+
+
+@pytest.mark.parametrize("name", ["one_centre", "small_weights", "across_faces", "box_of_a_particle", "many_centres",
+                                  "long_box"])
+@pytest.mark.parametrize("q", [15, 19])
+def test_ibb_link_distances_over_shapes(name, q):
+    """Binary64 storage, one step from the oracle's own state: the update depends on q of every link,
+    and a q off by one bisection bracket (6e-8) would move a population by some 1e-9 of the largest,
+    a thousand times the bound."""
+    _need_gpu()
+    from oracle.oracle import Oracle, lattice
+    from paper_2308_05007_gb300 import inputs as I
+    from paper_2308_05007_gb300.rwmi import Simulation
+    dims, walls, parts = _shapes(name)
+    rng = np.random.default_rng(4)
+    cb = [rng.normal(0.0, s, (n, 3)).astype(np.float32) for _, n, s, _ in parts]
+    k = [rng.uniform(*r, n).astype(np.float32) for _, n, _, r in parts]
+    P = len(parts)
+    mb = I.Metaballs(center_offsets=np.cumsum([0] + [len(v) for v in k]).astype(np.int32), centers_body=np.concatenate(cb),
+                     k=np.concatenate(k), origin=np.array([p[0] for p in parts]), amplitude=np.tile([1.5, 0.7, 0.4], (P, 1)),
+                     period=np.full(P, 150.0), phase=np.full(P, 0.3), omega=np.tile([0.002, 0.001, 0.004], (P, 1)))
+    w = I.Workload(name=name, dims=dims, tau=0.75, D=0.02, seed=1, q=q, wall_mask=walls, body_force=(2e-5, 5e-6, 0.0),
+                   metaballs=mb, storage=3, coupling=1)
+    with Simulation.from_workload(w, seed_walkers=False) as sim:
+        eg, _ = sim.lattice()
+        eo, _ = lattice(q)
+        perm = np.array([int(np.where((eg == eo[i]).all(1))[0][0]) for i in range(q)])
+        for steps in (3, 4):
+            sim.step(steps)
+            t, f_prev, u_prev = sim.t, sim.populations()[perm], sim.velocity().astype(np.float64)
+            sim.step(1)
+            f_gpu, F_gpu = sim.populations()[perm], sim.particle_forces()
+            ora = Oracle.from_workload(w, seed_walkers=False)
+            ora.set_populations(f_prev)
+            ora.set_velocity(u_prev)
+            ora.set_time(t)
+            ora.step_fluid(1)
+            f_ora, F_ora = ora.populations(), ora.forces()
+            assert np.abs(f_gpu - f_ora).max() <= 1e-12 * np.abs(f_ora).max()
+            assert np.abs(F_gpu - F_ora).max() <= 1e-9 * np.abs(F_ora).max()
+            assert np.abs(F_ora).max() > 0.0
