@@ -57,6 +57,8 @@ struct rwmi_ctx {
   rwmi_config cfg;
   Geom g;
   int device = 0, nsm = 152;
+  int nsm_part = 0;   // SMs this context's raster and resolve grids are sized for: all (0), or its part
+                      // when many contexts step concurrently (branches of a batch)
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   cudaStream_t side = nullptr;    // raster of t+1 beside the LBM of t
@@ -162,9 +164,8 @@ struct rwmi_batch {
   int mode = RWMI_BATCH_AUTO;
   bool fused = false;
   rwmi_batch_tiles tiles{128, 1, 8192, 64};
-  cudaStream_t side = nullptr;           // raster of t+1 beside the LBM of t
   cudaStream_t wst = nullptr;            // walkers of t beside the fluid of t+1
-  cudaEvent_t fork2 = nullptr, join2 = nullptr, fluid_ev = nullptr, walk_ev[2] = {nullptr, nullptr};
+  cudaEvent_t fluid_ev = nullptr, walk_ev[2] = {nullptr, nullptr};
   BlockMap* maps = nullptr;              // device: the block maps of every phase, back to back
   size_t map_off[FP_COUNT] = {}, map_n[FP_COUNT] = {};
   std::map<std::vector<int>, FusedGraph> fgraphs;
@@ -524,6 +525,7 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
   const int tp = (int)(c->t & 1), tn = tp ^ 1;
   const int toff = (int)(c->t - c->t_base);
   const ParticleSet ps = particle_set(c);
+  const int part = c->nsm_part > 0 ? c->nsm_part : c->nsm;
   const uint32_t k0 = (uint32_t)c->seed, k1 = (uint32_t)(c->seed >> 32);
   const int level = c->timing ? 0 : c->cfg.overlap;
   const bool fork_raster = level >= 1 && c->P > 0;
@@ -599,7 +601,7 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     lbm();
     pose();
     phase_begin(c, RWMI_PHASE_RASTER);
-    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->stream, classes);
+    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, part, c->stream, classes);
     c->launches++;
     phase_end(c, RWMI_PHASE_RASTER);
   } else if (fork_raster && !ibb && !(c->tma_ok && c->cfg.lbm_staging)) {
@@ -607,14 +609,14 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     // the update sometimes took every SM first, and the raster ran only as it drained (256^3: 707
     // to 768 us per step from one build to the next, 708 us in this order)
     pose();
-    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->stream);
+    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, part, c->stream);
     c->launches++;
     lbm(true);
   } else if (fork_raster) {
     pose();
     cudaEventRecord(c->fork_ev, c->stream);
     cudaStreamWaitEvent(c->side, c->fork_ev, 0);
-    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->side, classes);
+    launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, part, c->side, classes);
     c->launches++;
     cudaEventRecord(c->join_ev, c->side);
     lbm();
@@ -624,7 +626,7 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     pose();
     phase_begin(c, RWMI_PHASE_RASTER);
     if (c->P > 0) {
-      launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, c->nsm, c->stream, classes);
+      launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, part, c->stream, classes);
       c->launches++;
     }
     phase_end(c, RWMI_PHASE_RASTER);
@@ -637,7 +639,7 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
   phase_begin(c, RWMI_PHASE_WALKERS);
   if (c->nw > 0) {
     launch_walkers(c->g, ps, brick_set(c, tn), c->pos[c->pcur], c->nw, c->u[tp], c->d_T, toff, tp, (float)c->D,
-                   k0, k1, c->status, c->wlist, c->wlist_n, c->nsm, ws);
+                   k0, k1, c->status, c->wlist, c->wlist_n, c->nsm, part, ws);
     c->launches += 2;
   }
   phase_end(c, RWMI_PHASE_WALKERS);
@@ -1795,18 +1797,30 @@ rwmi_status fused_build_maps(rwmi_batch* b) {
     }
     b->map_n[phase] = all.size() - b->map_off[phase];
   };
+  // The tiles say how much work a block takes at most; where that leaves SMs empty (a few small
+  // domains), a domain's raster and resolve passes take their share of a full grid instead: their
+  // bricks and walkers then go to more warps (64 domains of 16^3-48^3: see the raster's pieces).
+  int64_t bricks = 1, walkers = 1;
+  for (const rwmi_ctx* c : b->ctxs) {
+    bricks += c->P > 0 ? c->nbrick : 0;
+    walkers += c->nw;
+  }
   const bool sorts = b->ctxs[0]->cfg.sort_interval > 0, moments = b->ctxs[0]->cfg.moment_interval > 0;
   add(FP_CLEARB, [&](rwmi_ctx* c) { return clear_grid(c->nbrick + BWORD_EXTRA); });
   add(FP_POSE, [&](rwmi_ctx* c) { return c->P > 0 ? c->P : 1; });
   add(FP_RASTER, [&](rwmi_ctx* c) {
-    return c->P > 0 ? std::min<int64_t>(std::max<int64_t>(ceil_div(c->nbrick, tl.raster_bricks_per_block), 1),
+    const int64_t share = 2 * raster_grid(c->nsm) * (int64_t)c->nbrick / bricks;   // four blocks fit an SM
+    return c->P > 0 ? std::min<int64_t>(std::max<int64_t>({ceil_div(c->nbrick, tl.raster_bricks_per_block), share, 1}),
                                         raster_grid(c->nsm))
                     : 0;
   });
   add(FP_LBM, [&](rwmi_ctx* c) { return ceil_div(c->ncell, tl.lbm_block); });
   add(FP_WALK, [&](rwmi_ctx* c) { return c->nw > 0 ? ceil_div(ceil_div(c->nw, 256), tl.walker_chunks_per_block) : 0; });
   add(FP_RESOLVE, [&](rwmi_ctx* c) {
-    return c->nw > 0 ? std::min<int64_t>(ceil_div(c->nw, tl.resolve_walkers_per_block), resolve_grid(c->nsm)) : 0;
+    const int64_t share = resolve_grid(c->nsm) * (int64_t)c->nw / walkers;
+    return c->nw > 0 ? std::min<int64_t>(std::max(ceil_div(c->nw, tl.resolve_walkers_per_block), share),
+                                         resolve_grid(c->nsm))
+                     : 0;
   });
   add(FP_CLEARC, [&](rwmi_ctx* c) { return sorts && c->nw > 0 ? clear_grid((uint32_t)c->ncell) : 0; });
   add(FP_HIST, [&](rwmi_ctx* c) { return sorts && c->nw > 0 ? ceil_div(c->nw, 256) : 0; });
@@ -1832,7 +1846,7 @@ rwmi_status fused_build_maps(rwmi_batch* b) {
 // Captures one chunk of L steps of every context as fused launches. The argument records of
 // every step are formed on the host while the host mirrors advance, exactly as enqueue_step
 // advances them, in its pipelined schedule: the raster of t+1 beside the LBM of t, and the
-// walkers of t (with the sort and moments) on a third stream beside the fluid of t+1; the fluid
+// walkers of t (with the sort and moments) on a second stream beside the fluid of t+1; the fluid
 // of t+2 waits for the walkers of t, the last readers of the buffers of that time parity.
 rwmi_status fused_capture(rwmi_batch* b, FusedGraph& fg) {
   const size_t ND = b->ctxs.size();
@@ -1917,21 +1931,18 @@ rwmi_status fused_capture(rwmi_batch* b, FusedGraph& fg) {
     if (walk_rec[par]) cudaStreamWaitEvent(b->origin, b->walk_ev[par], 0);
     launch_clear_batched(A(s, FP_CLEARB), M(FP_CLEARB), N(FP_CLEARB), b->origin); count(FP_CLEARB);
     launch_pose_batched(A(s, FP_POSE), M(FP_POSE), N(FP_POSE), b->origin); count(FP_POSE);
-    cudaEventRecord(b->fork2, b->origin);
-    cudaStreamWaitEvent(b->side, b->fork2, 0);
-    launch_raster_batched(A(s, FP_RASTER), M(FP_RASTER), N(FP_RASTER), b->side); count(FP_RASTER);
-    cudaEventRecord(b->join2, b->side);
+    // the update starts once the raster's blocks are resident, as in enqueue_step
+    launch_raster_batched(A(s, FP_RASTER), M(FP_RASTER), N(FP_RASTER), b->origin); count(FP_RASTER);
     // the FP64 sums on the chunk's last step, as in rwmi_step: the fused update-and-reduce pass
     // where the storage has one (same stored bits), else the update and a reduce-only pass
     const bool fuse = s == L - 1 && fused_storage(storage);
     launch_lbm_batched(q, storage, walls, fuse ? 2 : 0, A(s, FP_LBM), M(FP_LBM), N(FP_LBM), b->tiles.lbm_block,
-                       b->origin);
+                       b->origin, N(FP_RASTER) > 0);
     count(FP_LBM);
     if (s == L - 1 && !fuse) {
       launch_lbm_batched(q, storage, walls, 1, A(s, FP_LBM), M(FP_LBM), N(FP_LBM), b->tiles.lbm_block, b->origin);
       count(FP_LBM);
     }
-    cudaStreamWaitEvent(b->origin, b->join2, 0);
     cudaEventRecord(b->fluid_ev, b->origin);
     cudaStreamWaitEvent(b->wst, b->fluid_ev, 0);
     cudaStream_t ws = b->wst;
@@ -2010,15 +2021,12 @@ RWMI_API rwmi_status rwmi_batch_create(rwmi_batch** out, rwmi_ctx* const* ctxs, 
     }
   auto init = [&]() -> rwmi_status {
     BCK(cudaStreamCreateWithFlags(&b->origin, cudaStreamNonBlocking));
-    BCK(cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking));
     BCK(cudaStreamCreateWithFlags(&b->wst, cudaStreamNonBlocking));
     BCK(cudaEventCreateWithFlags(&b->fluid_ev, cudaEventDisableTiming));
     BCK(cudaEventCreateWithFlags(&b->walk_ev[0], cudaEventDisableTiming));
     BCK(cudaEventCreateWithFlags(&b->walk_ev[1], cudaEventDisableTiming));
     BCK(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
     BCK(cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming));
-    BCK(cudaEventCreateWithFlags(&b->fork2, cudaEventDisableTiming));
-    BCK(cudaEventCreateWithFlags(&b->join2, cudaEventDisableTiming));
     b->join.resize(b->ctxs.size());
     for (auto& e : b->join) BCK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     return RWMI_OK;
@@ -2064,7 +2072,11 @@ RWMI_API rwmi_status rwmi_batch_step(rwmi_batch* b, int32_t nsteps) try {
       for (size_t k = 0; k < b->ctxs.size(); ++k) {
         rwmi_ctx* c = b->ctxs[k];
         cudaStreamWaitEvent(c->stream, b->fork, 0);
+        // Grids that fill the chip for one context only add work for many at a time (a raster cut into
+        // more pieces; 24 domains of 48^3-120^3: 1370 us per step, 1080 us with a part each).
+        c->nsm_part = std::max(8, c->nsm / (int)b->ctxs.size());
         for (int64_t st = 0; st < b->L; ++st) enqueue_step(c, st == b->L - 1);
+        c->nsm_part = 0;
         segment_end(c);
         cudaEventRecord(b->join[k], c->stream);
         cudaStreamWaitEvent(b->origin, b->join[k], 0);
@@ -2121,12 +2133,9 @@ RWMI_API void rwmi_batch_destroy(rwmi_batch* b) {
   for (auto e : b->join) if (e) cudaEventDestroy(e);
   if (b->fork) cudaEventDestroy(b->fork);
   if (b->done) cudaEventDestroy(b->done);
-  if (b->fork2) cudaEventDestroy(b->fork2);
-  if (b->join2) cudaEventDestroy(b->join2);
   if (b->fluid_ev) cudaEventDestroy(b->fluid_ev);
   if (b->walk_ev[0]) cudaEventDestroy(b->walk_ev[0]);
   if (b->walk_ev[1]) cudaEventDestroy(b->walk_ev[1]);
-  if (b->side) cudaStreamDestroy(b->side);
   if (b->wst) cudaStreamDestroy(b->wst);
   if (b->origin) cudaStreamDestroy(b->origin);
   delete b;

@@ -787,6 +787,7 @@ __global__ void __launch_bounds__(256, 4) raster_kernel(const RasterArgs a) {
 }
 __global__ void __launch_bounds__(256, 4) raster_batched(const RasterArgs* __restrict__ args,
                                                          const BlockMap* __restrict__ map) {
+  asm volatile("griddepcontrol.launch_dependents;");   // as raster_kernel
   const BlockMap m = map[blockIdx.x];
   raster_body(args[m.domain], m.block, m.blocks);
 }

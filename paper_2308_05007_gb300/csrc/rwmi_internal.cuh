@@ -159,27 +159,7 @@ __device__ __forceinline__ float metaball_exact(const float4* __restrict__ cw, i
   return f;
 }
 
-// Eq. 3 and Eq. 17 for walker decisions (binary32, contraction and fast reciprocals allowed).
-__device__ __forceinline__ float metaball_grad(const float4* __restrict__ cw, int c0, int c1,
-                                               float x, float y, float z, const Geom& g,
-                                               float* gx, float* gy, float* gz) {
-  float f = 0.0f, ax = 0.0f, ay = 0.0f, az = 0.0f;
-  for (int i = c0; i < c1; ++i) {
-    const float4 c = cw[i];
-    const float dx = min_image_rn(x - c.x, (float)g.n[0], g.wall[0]);
-    const float dy = min_image_rn(y - c.y, (float)g.n[1], g.wall[1]);
-    const float dz = min_image_rn(z - c.z, (float)g.n[2], g.wall[2]);
-    const float r2 = dx * dx + dy * dy + dz * dz;
-    const float inv = __frcp_rn(r2);
-    const float term = c.w * inv;
-    f += term;
-    const float s = -2.0f * term * inv;
-    ax += s * dx; ay += s * dy; az += s * dz;
-  }
-  if (gx) { *gx = ax; *gy = ay; *gz = az; }
-  return f;
-}
-
+// Eq. 3 for decisions that need no exact rounding (binary32, contraction and fast quotients allowed).
 __device__ __forceinline__ float metaball_value(const float4* __restrict__ cw, int c0, int c1,
                                                 float x, float y, float z, const Geom& g) {
   float f = 0.0f;
@@ -368,7 +348,7 @@ inline int64_t wlist_stripe_cap(int64_t n) {
 void launch_walkers(const Geom& g, const ParticleSet& ps, BrickSet bs1, float4* pos, int64_t n,
                     const float* u, const int64_t* d_T, int toff, int toff_parity, float D,
                     uint32_t k0, uint32_t k1, unsigned long long* status, float4* list,
-                    unsigned int* list_n, int nsm, cudaStream_t st);
+                    unsigned int* list_n, int nsm, int nsm_resolve, cudaStream_t st);
 void launch_advance(int64_t* d_T, int64_t k, cudaStream_t st);
 void launch_seed(const Geom& g, const ParticleSet& ps, BrickSet bs, float4* pos, float4* x0,
                  int64_t n, const double lo[3], const double hi[3], uint32_t k0, uint32_t k1,
@@ -427,7 +407,8 @@ void lbm_args(void* dst, int q, int storage, const Geom& g, const void* fin, voi
               const uint16_t* solid, BrickSet bs, double tau, double rho0, double* red, double* forces);
 // mode 0 the update, 1 the reduce-only pass, 2 both in one pass (binary32-shifted and binary64)
 void launch_lbm_batched(int q, int storage, bool walls, int mode, const void* args, const BlockMap* map,
-                        int nblocks, int block, cudaStream_t st);
+                        int nblocks, int block, cudaStream_t st,
+                        bool after_raster = false);
 size_t walker_args_size();
 void walker_args(void* dst, const Geom& g, const ParticleSet& ps, BrickSet bs1, float4* pos, int64_t n,
                  const float* u, const int64_t* d_T, int toff, int toff_parity, float D, uint32_t k0,

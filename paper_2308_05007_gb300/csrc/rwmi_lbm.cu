@@ -708,6 +708,7 @@ __global__ void __launch_bounds__(256, sizeof(typename Store<STORE>::R) == 8 ? 2
   lbm_body<Q, STORE, WALLS, MODE, IBB>(a.g, a.pl, a.u4, a.solid, a.bword, a.pose, a.posed, a.sp, a.tau, a.omega,
                                        a.guo0, a.rho0, a.red, a.forces, nullptr, nullptr, nullptr, nullptr,
                                        nullptr, nullptr, nullptr, nullptr, 0, nullptr, m.block);
+  if (blockIdx.x == gridDim.x - 1) asm volatile("griddepcontrol.wait;" ::: "memory");   // as lbm_kernel
 }
 #undef RWMI_LBM_BOUNDS
 
@@ -1291,29 +1292,29 @@ void lbm_args(void* dst, int q, int storage, const Geom& g, const void* fin, voi
 
 template <int Q, int STORE>
 static void launch_lbm_batched_q(bool walls, int mode, const void* args, const BlockMap* map, int nblocks, int block,
-                                 cudaStream_t st) {
+                                 cudaStream_t st, bool after_raster) {
   const LbmArgs<Q, STORE>* a = static_cast<const LbmArgs<Q, STORE>*>(args);
   if constexpr (STORE == 1 || STORE == 3) {   // the fused update and reduction
     if (mode == 2) {
-      if (walls) lbm_batched<Q, STORE, true, 2, false><<<nblocks, block, 0, st>>>(a, map);
-      else lbm_batched<Q, STORE, false, 2, false><<<nblocks, block, 0, st>>>(a, map);
+      if (walls) launch_kernel(lbm_batched<Q, STORE, true, 2, false>, nblocks, block, st, after_raster, a, map);
+      else launch_kernel(lbm_batched<Q, STORE, false, 2, false>, nblocks, block, st, after_raster, a, map);
       return;
     }
   }
   if (walls) {
-    if (mode == 0) lbm_batched<Q, STORE, true, 0, false><<<nblocks, block, 0, st>>>(a, map);
+    if (mode == 0) launch_kernel(lbm_batched<Q, STORE, true, 0, false>, nblocks, block, st, after_raster, a, map);
     else lbm_batched<Q, STORE, true, 1, false><<<nblocks, block, 0, st>>>(a, map);
   } else {
-    if (mode == 0) lbm_batched<Q, STORE, false, 0, false><<<nblocks, block, 0, st>>>(a, map);
+    if (mode == 0) launch_kernel(lbm_batched<Q, STORE, false, 0, false>, nblocks, block, st, after_raster, a, map);
     else lbm_batched<Q, STORE, false, 1, false><<<nblocks, block, 0, st>>>(a, map);
   }
 }
 
 void launch_lbm_batched(int q, int storage, bool walls, int mode, const void* args, const BlockMap* map,
-                        int nblocks, int block, cudaStream_t st) {
+                        int nblocks, int block, cudaStream_t st, bool after_raster) {
   if (nblocks <= 0) return;
   block = (block == 64 || block == 128) ? block : 256;
-#define RWMI_LB(QQ, SS) launch_lbm_batched_q<QQ, SS>(walls, mode, args, map, nblocks, block, st)
+#define RWMI_LB(QQ, SS) launch_lbm_batched_q<QQ, SS>(walls, mode, args, map, nblocks, block, st, after_raster)
   if (q == 15) {
     if (storage == 0) RWMI_LB(15, 0); else if (storage == 1) RWMI_LB(15, 1);
     else if (storage == 2) RWMI_LB(15, 2); else RWMI_LB(15, 3);

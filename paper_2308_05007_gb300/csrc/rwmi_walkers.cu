@@ -99,68 +99,119 @@ struct WalkCtx {
   BrickSet bs;
 };
 
-__device__ __forceinline__ float f_particle(const WalkCtx& c, int p, const float* x, float* gr) {
-  const float xw = wrap_coord(x[0], (float)c.g.n[0], c.g.wall[0], c.g.inv_n[0]);
-  const float yw = wrap_coord(x[1], (float)c.g.n[1], c.g.wall[1], c.g.inv_n[1]);
-  const float zw = wrap_coord(x[2], (float)c.g.n[2], c.g.wall[2], c.g.inv_n[2]);
-  const ParticleDesc& d = c.ps.desc[p];
-  if (gr) return metaball_grad(c.bs.cworld, d.c0, d.c1, xw, yw, zw, c.g, gr, gr + 1, gr + 2);
-  return metaball_value(c.bs.cworld, d.c0, d.c1, xw, yw, zw, c.g);
+// ---- a walker that meets a particle, resolved by one warp ------------------------------------
+// Every lane holds the walker; Eq. 3's terms are formed by one lane per control point (kept in its
+// registers while one particle is asked again and again) and summed by all in control point
+// order, so a value is that of a loop over the points, bit for bit. Algorithm 1 and the refill
+// are chains of some fifteen values: with a loop per lane, a load and a quotient deep per control
+// point, they were most of the resolve pass.
+struct WarpParticle {
+  int p, c0, c1;   // the particle held, its control points
+  float4 c;        // this lane's: c0 + lane
+};
+__device__ __forceinline__ void hold(const WalkCtx& c, int p, WarpParticle& h) {
+  if (h.p == p) return;
+  h.p = p;
+  h.c0 = c.ps.desc[p].c0;
+  h.c1 = c.ps.desc[p].c1;
+  const int lane = threadIdx.x & 31;
+  if (h.c0 + lane < h.c1) h.c = c.bs.cworld[h.c0 + lane];
 }
-
-// Lowest-index particle holding x (any particle; bound-radius skip), or -1.
-__device__ int inside_any(const WalkCtx& c, const float* x) {
-  const float xw = wrap_coord(x[0], (float)c.g.n[0], c.g.wall[0], c.g.inv_n[0]);
-  const float yw = wrap_coord(x[1], (float)c.g.n[1], c.g.wall[1], c.g.inv_n[1]);
-  const float zw = wrap_coord(x[2], (float)c.g.n[2], c.g.wall[2], c.g.inv_n[2]);
-  for (int p = 0; p < c.ps.P; ++p) {
-    const PoseF& pp = c.bs.pose[p];
-    const float dx = min_image_rn(xw - pp.o[0], (float)c.g.n[0], c.g.wall[0]);
-    const float dy = min_image_rn(yw - pp.o[1], (float)c.g.n[1], c.g.wall[1]);
-    const float dz = min_image_rn(zw - pp.o[2], (float)c.g.n[2], c.g.wall[2]);
-    const float rb = c.ps.desc[p].rb + 1e-3f;
-    if (dx * dx + dy * dy + dz * dz > rb * rb) continue;
-    const ParticleDesc& d = c.ps.desc[p];
-    if (metaball_value(c.bs.cworld, d.c0, d.c1, xw, yw, zw, c.g) >= 1.0f) return p;
+// a^2 + b^2 + c^2 and its like with the multiply-adds written out: this rounding, since a walker's new
+// position carries it
+__device__ __forceinline__ float dot3(float a0, float a1, float a2, float b0, float b1, float b2) {
+  return fmaf(a2, b2, fmaf(a0, b0, __fmul_rn(a1, b1)));
+}
+__device__ __forceinline__ float square3(float a, float b, float c) { return dot3(a, b, c, a, b, c); }
+struct Wrapped { float x, y, z; };
+__device__ __forceinline__ Wrapped wrapped(const WalkCtx& c, const float* x) {
+  return Wrapped{wrap_coord(x[0], (float)c.g.n[0], c.g.wall[0], c.g.inv_n[0]),
+                 wrap_coord(x[1], (float)c.g.n[1], c.g.wall[1], c.g.inv_n[1]),
+                 wrap_coord(x[2], (float)c.g.n[2], c.g.wall[2], c.g.inv_n[2])};
+}
+// Eq. 3 of the particle held, at a wrapped point: k times the fast reciprocal of r^2, added with one
+// rounding
+__device__ __forceinline__ float warp_value(const WalkCtx& c, const WarpParticle& h, const Wrapped& w) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  float f = 0.0f;
+  for (int base = h.c0; base < h.c1; base += 32) {
+    const int n = min(h.c1 - base, 32);
+    float k = 0.0f, inv = 0.0f;
+    if (lane < n) {
+      const float4 cc = base == h.c0 ? h.c : c.bs.cworld[base + lane];
+      const float dx = min_image_rn(w.x - cc.x, (float)c.g.n[0], c.g.wall[0]);
+      const float dy = min_image_rn(w.y - cc.y, (float)c.g.n[1], c.g.wall[1]);
+      const float dz = min_image_rn(w.z - cc.z, (float)c.g.n[2], c.g.wall[2]);
+      k = cc.w;
+      asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(square3(dx, dy, dz)));
+    }
+    for (int i = 0; i < n; ++i) f = fmaf(__shfl_sync(full, k, i), __shfl_sync(full, inv, i), f);
   }
-  return -1;
+  return f;
+}
+// Its gradient, Eq. 17: the sum of -2 k (x - c) / r^4.
+__device__ __forceinline__ void warp_grad(const WalkCtx& c, const WarpParticle& h, const Wrapped& w, float* gr) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  float ax = 0.0f, ay = 0.0f, az = 0.0f;
+  for (int base = h.c0; base < h.c1; base += 32) {
+    const int n = min(h.c1 - base, 32);
+    float s = 0.0f, dx = 0.0f, dy = 0.0f, dz = 0.0f;
+    if (lane < n) {
+      const float4 cc = base == h.c0 ? h.c : c.bs.cworld[base + lane];
+      dx = min_image_rn(w.x - cc.x, (float)c.g.n[0], c.g.wall[0]);
+      dy = min_image_rn(w.y - cc.y, (float)c.g.n[1], c.g.wall[1]);
+      dz = min_image_rn(w.z - cc.z, (float)c.g.n[2], c.g.wall[2]);
+      const float inv = __frcp_rn(square3(dx, dy, dz));
+      s = -2.0f * (cc.w * inv) * inv;
+    }
+    for (int i = 0; i < n; ++i) {
+      const float si = __shfl_sync(full, s, i);
+      ax = fmaf(si, __shfl_sync(full, dx, i), ax);
+      ay = fmaf(si, __shfl_sync(full, dy, i), ay);
+      az = fmaf(si, __shfl_sync(full, dz, i), az);
+    }
+  }
+  gr[0] = ax; gr[1] = ay; gr[2] = az;
+}
+__device__ __forceinline__ bool beyond_bound(const WalkCtx& c, int p, const Wrapped& w) {
+  const PoseF& pp = c.bs.pose[p];
+  const float dx = min_image_rn(w.x - pp.o[0], (float)c.g.n[0], c.g.wall[0]);
+  const float dy = min_image_rn(w.y - pp.o[1], (float)c.g.n[1], c.g.wall[1]);
+  const float dz = min_image_rn(w.z - pp.o[2], (float)c.g.n[2], c.g.wall[2]);
+  const float rb = c.ps.desc[p].rb + 1e-3f;
+  return dx * dx + dy * dy + dz * dz > rb * rb;
 }
 
-// inside_any through the candidate list of x's own brick: a particle holding x lies within its
-// bound radius of x, so it is on that list (built at the same time with a larger radius). Same
-// answer (lowest index), a handful of particles instead of all; all of them when the list
-// overflowed.
-__device__ int inside_cand(const WalkCtx& c, const float* x) {
-  const float xw = wrap_coord(x[0], (float)c.g.n[0], c.g.wall[0], c.g.inv_n[0]);
-  const float yw = wrap_coord(x[1], (float)c.g.n[1], c.g.wall[1], c.g.inv_n[1]);
-  const float zw = wrap_coord(x[2], (float)c.g.n[2], c.g.wall[2], c.g.inv_n[2]);
-  const int b = brick_of(xw, yw, zw, c.g);
+// Lowest-index particle holding x, or -1, through the candidate list of x's own brick: a particle
+// holding x lies within its bound radius of x, so it is on that list (built at the same time with a
+// larger radius); all particles when the list overflowed.
+__device__ int inside_cand(const WalkCtx& c, WarpParticle& h, const float* x) {
+  const Wrapped w = wrapped(c, x);
+  const int b = brick_of(w.x, w.y, w.z, c.g);
   const uint32_t nc = c.bs.bword[b] & 0xffffu;
-  if (nc > MAXC) return inside_any(c, x);
+  const bool all = nc > MAXC;
+  const uint32_t n = all ? (uint32_t)c.ps.P : nc;
   int best = -1;
-  for (uint32_t m = 0; m < nc; ++m) {
-    const int p = c.bs.bcand[b * MAXC + m] & 0x7fff;
+  for (uint32_t m = 0; m < n; ++m) {
+    const int p = all ? (int)m : (c.bs.bcand[b * MAXC + m] & 0x7fff);
     if (best >= 0 && p > best) continue;
-    const PoseF& pp = c.bs.pose[p];
-    const float dx = min_image_rn(xw - pp.o[0], (float)c.g.n[0], c.g.wall[0]);
-    const float dy = min_image_rn(yw - pp.o[1], (float)c.g.n[1], c.g.wall[1]);
-    const float dz = min_image_rn(zw - pp.o[2], (float)c.g.n[2], c.g.wall[2]);
-    const float rb = c.ps.desc[p].rb + 1e-3f;
-    if (dx * dx + dy * dy + dz * dz > rb * rb) continue;
-    const ParticleDesc& d = c.ps.desc[p];
-    if (metaball_value(c.bs.cworld, d.c0, d.c1, xw, yw, zw, c.g) >= 1.0f) best = p;
+    if (beyond_bound(c, p, w)) continue;
+    hold(c, p, h);
+    if (warp_value(c, h, w) >= 1.0f) best = p;
   }
   return best;
 }
 
-// Algorithm 1: bisection from outside point a (f < 1) to inside point b (f >= 1) of particle p;
+// Algorithm 1: bisection from outside point a (f < 1) to inside point b (f >= 1) of the particle held;
 // |f(mid) - 1| < 1e-3 converges; at most 200 iterations. aout: final outside end.
-__device__ bool bisect(const WalkCtx& c, int p, const float* a_in, const float* b_in, float* xi, float* aout) {
+__device__ bool bisect(const WalkCtx& c, const WarpParticle& h, const float* a_in, const float* b_in, float* xi, float* aout) {
   float a[3] = {a_in[0], a_in[1], a_in[2]}, b[3] = {b_in[0], b_in[1], b_in[2]};
   bool found = false;
   for (int it = 1; it <= 200; ++it) {
     float mid[3] = {0.5f * (a[0] + b[0]), 0.5f * (a[1] + b[1]), 0.5f * (a[2] + b[2])};
-    const float fm = f_particle(c, p, mid, nullptr);
+    const float fm = warp_value(c, h, wrapped(c, mid));
     if (fabsf(fm - 1.0f) < 1e-3f) {
       xi[0] = mid[0]; xi[1] = mid[1]; xi[2] = mid[2];
       found = true;
@@ -175,26 +226,27 @@ __device__ bool bisect(const WalkCtx& c, int p, const float* a_in, const float* 
   return found;
 }
 
-// Section 2.4.2 refill of a type-II walker (see the oracle's reading, implemented alike).
-__device__ bool refill(const WalkCtx& c, int p, const float* x, uint32_t id, uint32_t t, float amp,
+// Section 2.4.2 refill of a type-II walker of particle p (see the oracle's reading, implemented alike).
+__device__ bool refill(const WalkCtx& c, WarpParticle& h, int p, const float* x, uint32_t id, uint32_t t, float amp,
                        uint32_t k0, uint32_t k1, float* xnew) {
+  hold(c, p, h);
   float gr[3];
-  f_particle(c, p, x, gr);
-  const float gn = sqrtf(gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2]);
+  warp_grad(c, h, wrapped(c, x), gr);
+  const float gn = sqrtf(square3(gr[0], gr[1], gr[2]));
   float s[3] = {1.0f, 0.0f, 0.0f};
   if (gn > 0.0f && isfinite(gn)) { s[0] = -gr[0] / gn; s[1] = -gr[1] / gn; s[2] = -gr[2] / gn; }
   float xo[3];
   bool out = false;
-  for (float h = 0.5f; h <= 64.0f; h *= 2.0f) {
-    xo[0] = x[0] + h * s[0]; xo[1] = x[1] + h * s[1]; xo[2] = x[2] + h * s[2];
-    if (f_particle(c, p, xo, nullptr) < 1.0f) { out = true; break; }
+  for (float hh = 0.5f; hh <= 64.0f; hh *= 2.0f) {
+    xo[0] = x[0] + hh * s[0]; xo[1] = x[1] + hh * s[1]; xo[2] = x[2] + hh * s[2];
+    if (warp_value(c, h, wrapped(c, xo)) < 1.0f) { out = true; break; }
   }
   if (!out) { xnew[0] = x[0]; xnew[1] = x[1]; xnew[2] = x[2]; return false; }
   float xs[3], aend[3];
-  if (!bisect(c, p, xo, x, xs, aend)) { xs[0] = aend[0]; xs[1] = aend[1]; xs[2] = aend[2]; }
+  if (!bisect(c, h, xo, x, xs, aend)) { xs[0] = aend[0]; xs[1] = aend[1]; xs[2] = aend[2]; }
   float gs[3];
-  f_particle(c, p, xs, gs);
-  const float gsn = sqrtf(gs[0] * gs[0] + gs[1] * gs[1] + gs[2] * gs[2]);
+  warp_grad(c, h, wrapped(c, xs), gs);
+  const float gsn = sqrtf(square3(gs[0], gs[1], gs[2]));
   const float no[3] = {-gs[0] / gsn, -gs[1] / gsn, -gs[2] / gsn};
   const uint4 r = philox(make_uint4(id, t, 1u, 0u), k0, k1);
   const float ct = 2.0f * uniform24(r.x) - 1.0f;
@@ -204,64 +256,63 @@ __device__ bool refill(const WalkCtx& c, int p, const float* x, uint32_t id, uin
   const float rad = amp * cbrtf(uniform24(r.z));
   float xr[3] = {xs[0] + rad * st * cp, xs[1] + rad * st * sp, xs[2] + rad * ct};
   wall_reflect(xr, c.g);
-  if (inside_cand(c, xr) >= 0) {
+  if (inside_cand(c, h, xr) >= 0) {
     const float dn = (xr[0] - xs[0]) * no[0] + (xr[1] - xs[1]) * no[1] + (xr[2] - xs[2]) * no[2];
     if (dn < 0.0f) for (int a = 0; a < 3; ++a) xr[a] -= 2.0f * dn * no[a];
     wall_reflect(xr, c.g);
-    if (inside_cand(c, xr) >= 0) {
+    if (inside_cand(c, h, xr) >= 0) {
       xr[0] = aend[0]; xr[1] = aend[1]; xr[2] = aend[2];
-      if (inside_cand(c, xr) >= 0) { xnew[0] = xr[0]; xnew[1] = xr[1]; xnew[2] = xr[2]; return false; }
+      if (inside_cand(c, h, xr) >= 0) { xnew[0] = xr[0]; xnew[1] = xr[1]; xnew[2] = xr[2]; return false; }
     }
   }
   xnew[0] = xr[0]; xnew[1] = xr[1]; xnew[2] = xr[2];
   return true;
 }
 
-// Rare path of a walker step (kept out of line so the common path keeps its registers): types
-// II-IV against the particles at t+1 (candidates of the walker's brick, or all particles when the
-// list overflowed or the step was unusually long). Returns event bits: 1 II, 2 III, 4 IV,
-// 8 Algorithm 1 failure, 16 refill failure; writes the new position to xn.
-__device__ __noinline__ unsigned resolve_particles(const WalkCtx& c, const float* x, const float* xf, float xw,
-                                                   float yw, float zw, int b, uint32_t nc, bool far_step,
-                                                   uint32_t id, uint32_t T, float amp, uint32_t k0, uint32_t k1,
-                                                   float* xn) {
+// Types II-IV of one walker (x to x_f) against the particles at t+1: candidates of the walker's brick
+// b, or all particles when the list overflowed or the step was unusually long. Returns event
+// bits: 1 II, 2 III, 4 IV, 8 Algorithm 1 failure, 16 refill failure; writes the new position to xn.
+__device__ unsigned resolve_particles(const WalkCtx& c, const float* x, const float* xf, const Wrapped& xw, int b,
+                                      uint32_t nc, bool far_step, uint32_t id, uint32_t T, float amp, uint32_t k0,
+                                      uint32_t k1, float* xn) {
   unsigned ev = 0u;
   int pin = -1, qin = -1;
+  WarpParticle h;
+  h.p = -1;
   if (nc > MAXC || far_step) {
-    pin = inside_cand(c, x);
-    qin = inside_cand(c, xf);
+    pin = inside_cand(c, h, x);
+    qin = inside_cand(c, h, xf);
   } else {
-    const float xfw = wrap_coord(xf[0], (float)c.g.n[0], c.g.wall[0], c.g.inv_n[0]);
-    const float yfw = wrap_coord(xf[1], (float)c.g.n[1], c.g.wall[1], c.g.inv_n[1]);
-    const float zfw = wrap_coord(xf[2], (float)c.g.n[2], c.g.wall[2], c.g.inv_n[2]);
+    const Wrapped xfw = wrapped(c, xf);
     for (uint32_t m = 0; m < nc; ++m) {
       const int p = c.bs.bcand[b * MAXC + m] & 0x7fff;
-      const ParticleDesc& d = c.ps.desc[p];
-      if ((pin < 0 || p < pin) && metaball_value(c.bs.cworld, d.c0, d.c1, xw, yw, zw, c.g) >= 1.0f) pin = p;
-      if ((qin < 0 || p < qin) && metaball_value(c.bs.cworld, d.c0, d.c1, xfw, yfw, zfw, c.g) >= 1.0f) qin = p;
+      hold(c, p, h);
+      if ((pin < 0 || p < pin) && warp_value(c, h, xw) >= 1.0f) pin = p;
+      if ((qin < 0 || p < qin) && warp_value(c, h, xfw) >= 1.0f) qin = p;
     }
   }
   if (pin >= 0 && qin >= 0) {            // type II: Dirichlet refill
     ev |= 1u;
-    if (!refill(c, pin, x, id, T, amp, k0, k1, xn)) ev |= 16u;
+    if (!refill(c, h, pin, x, id, T, amp, k0, k1, xn)) ev |= 16u;
   } else if (pin >= 0) {                 // type III: moves out freely
     ev |= 2u;
   } else if (qin >= 0) {                 // type IV: Algorithms 1 and 2
     ev |= 4u;
     float xi[3];
-    if (!bisect(c, qin, x, xf, xi, nullptr)) {
+    hold(c, qin, h);
+    if (!bisect(c, h, x, xf, xi, nullptr)) {
       ev |= 8u;
       xn[0] = x[0]; xn[1] = x[1]; xn[2] = x[2];
     } else {
       float gr[3];
-      f_particle(c, qin, xi, gr);
-      const float gn = sqrtf(gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2]);
+      warp_grad(c, h, wrapped(c, xi), gr);
+      const float gn = sqrtf(square3(gr[0], gr[1], gr[2]));
       const float nv[3] = {gr[0] / gn, gr[1] / gn, gr[2] / gn};
       const float ti[3] = {xf[0] - xi[0], xf[1] - xi[1], xf[2] - xi[2]};
-      const float tn = ti[0] * nv[0] + ti[1] * nv[1] + ti[2] * nv[2];
+      const float tn = dot3(ti[0], ti[1], ti[2], nv[0], nv[1], nv[2]);
       float tr[3];
       for (int a = 0; a < 3; ++a) tr[a] = xi[a] + (ti[a] - 2.0f * tn * nv[a]);
-      if (beyond_wall(tr, c.g) || inside_cand(c, tr) >= 0) {
+      if (beyond_wall(tr, c.g) || inside_cand(c, h, tr) >= 0) {
         xn[0] = x[0]; xn[1] = x[1]; xn[2] = x[2];
       } else {
         xn[0] = tr[0]; xn[1] = tr[1]; xn[2] = tr[2];
@@ -412,8 +463,10 @@ __device__ __forceinline__ void walker_body(const WalkCtx& c, float4* __restrict
 }
 
 // Pass 2 (fixed grid, grid-stride over the list stripes taken as one sequence): types II-IV of
-// the flagged walkers, written back to their slots. Block 0 clears the other parity's counters,
-// which the next step's pass 1 appends to.
+// the flagged walkers, written back to their slots. A thread per walker tests x and x_f against the
+// candidates; the few that meet a particle (~2%) queue up in shared memory and take a warp each. Block
+// 0 clears the other parity's counters, which the next step's pass 1 appends to.
+constexpr int RESOLVE_THREADS = 128;
 __device__ __forceinline__ void resolve_body(const WalkCtx& c, float4* __restrict__ pos,
                                              const float4* __restrict__ list, const unsigned int* list_n,
                                              unsigned int* list_n_next, const int64_t* d_T, int toff, float amp,
@@ -422,6 +475,8 @@ __device__ __forceinline__ void resolve_body(const WalkCtx& c, float4* __restric
   const int64_t T = *d_T + toff;
   // the stripes as one sequence: s_pre[k] = entries in stripes before k (first warp's scan)
   __shared__ unsigned s_pre[WLIST_STRIPES + 1];
+  __shared__ size_t s_hit[RESOLVE_THREADS];   // list slots of the walkers that meet a particle
+  __shared__ unsigned s_nhit;
   static_assert(WLIST_STRIPES == 32, "one lane per stripe");
   if (threadIdx.x < 32) {
     const unsigned v = list_n[threadIdx.x];
@@ -438,70 +493,83 @@ __device__ __forceinline__ void resolve_body(const WalkCtx& c, float4* __restric
       list_n_next[threadIdx.x] = 0u;   // the next step's counters (nobody reads them now)
     }
   }
+  if (threadIdx.x == 0) s_nhit = 0u;
   __syncthreads();
   const unsigned total = s_pre[WLIST_STRIPES];
   unsigned ev_all[5] = {0u, 0u, 0u, 0u, 0u};
-  const unsigned stride = nblk * blockDim.x;
-  for (unsigned e = blk * blockDim.x + threadIdx.x; e < total; e += stride) {
-    // stripe of entry e: the last k with s_pre[k] <= e, by bisection over the power-of-two
-    // stripe count (k < WLIST_STRIPES since e < total = s_pre[WLIST_STRIPES])
-    static_assert((WLIST_STRIPES & (WLIST_STRIPES - 1)) == 0, "stripe count must be a power of two");
-    int k = 0;
+  // walkers per block and turn: a short list is dealt out 32 at a time, so that its hits find more warps
+  const unsigned share = (total + (unsigned)nblk - 1u) / (unsigned)nblk;
+  const unsigned per = share >= RESOLVE_THREADS ? RESOLVE_THREADS : (share + 31u) & ~31u;
+  for (unsigned e0 = blk * per; e0 < total; e0 += nblk * per) {
+    const unsigned e = e0 + threadIdx.x;
+    if (threadIdx.x < per && e < total) {
+      // stripe of entry e: the last k with s_pre[k] <= e, by bisection over the power-of-two
+      // stripe count (k < WLIST_STRIPES since e < total = s_pre[WLIST_STRIPES])
+      static_assert((WLIST_STRIPES & (WLIST_STRIPES - 1)) == 0, "stripe count must be a power of two");
+      int k = 0;
 #pragma unroll
-    for (int half = WLIST_STRIPES / 2; half > 0; half >>= 1)
-      if (s_pre[k + half] <= e) k += half;
-    const size_t slot = (size_t)k * (size_t)cap + (e - s_pre[k]);
-    const float4 a = list[2 * slot], bq = list[2 * slot + 1];
-    const float x[3] = {a.x, a.y, a.z}, xf[3] = {bq.x, bq.y, bq.z};
-    const uint32_t id = __float_as_uint(a.w);
-    const uint32_t w = __float_as_uint(bq.w);
-    const float xw = wrap_coord(x[0], (float)c.g.n[0], c.g.wall[0], c.g.inv_n[0]);
-    const float yw = wrap_coord(x[1], (float)c.g.n[1], c.g.wall[1], c.g.inv_n[1]);
-    const float zw = wrap_coord(x[2], (float)c.g.n[2], c.g.wall[2], c.g.inv_n[2]);
-    const int b = brick_of(xw, yw, zw, c.g);
-    const uint32_t nc = c.bs.bword[b] & 0xffffu;
-    const float step2 = (xf[0] - x[0]) * (xf[0] - x[0]) + (xf[1] - x[1]) * (xf[1] - x[1]) +
-                        (xf[2] - x[2]) * (xf[2] - x[2]);
-    const bool far_step = step2 > c.ps.walk_margin * c.ps.walk_margin;
-    float xn[3] = {xf[0], xf[1], xf[2]};
-    // most flagged walkers meet no particle: test x and x_f against the brick's candidates inline
-    // (one pass over each candidate's control points) and take the out-of-line path only on a hit
-    bool hit = far_step || nc > MAXC;
-    if (!hit) {
-      const float xfw = wrap_coord(xf[0], (float)c.g.n[0], c.g.wall[0], c.g.inv_n[0]);
-      const float yfw = wrap_coord(xf[1], (float)c.g.n[1], c.g.wall[1], c.g.inv_n[1]);
-      const float zfw = wrap_coord(xf[2], (float)c.g.n[2], c.g.wall[2], c.g.inv_n[2]);
-      for (uint32_t m = 0; m < nc && !hit; ++m) {
-        const ParticleDesc& d = c.ps.desc[c.bs.bcand[b * MAXC + m] & 0x7fff];
-        float fa = 0.0f, fb = 0.0f;
-        for (int i = d.c0; i < d.c1; ++i) {
-          const float4 cc = c.bs.cworld[i];
-          const float ax = min_image_rn(xw - cc.x, (float)c.g.n[0], c.g.wall[0]);
-          const float ay = min_image_rn(yw - cc.y, (float)c.g.n[1], c.g.wall[1]);
-          const float az = min_image_rn(zw - cc.z, (float)c.g.n[2], c.g.wall[2]);
-          const float bx = min_image_rn(xfw - cc.x, (float)c.g.n[0], c.g.wall[0]);
-          const float by = min_image_rn(yfw - cc.y, (float)c.g.n[1], c.g.wall[1]);
-          const float bz = min_image_rn(zfw - cc.z, (float)c.g.n[2], c.g.wall[2]);
-          fa += __fdividef(cc.w, ax * ax + ay * ay + az * az);
-          fb += __fdividef(cc.w, bx * bx + by * by + bz * bz);
+      for (int half = WLIST_STRIPES / 2; half > 0; half >>= 1)
+        if (s_pre[k + half] <= e) k += half;
+      const size_t slot = (size_t)k * (size_t)cap + (e - s_pre[k]);
+      const float4 a = list[2 * slot], bq = list[2 * slot + 1];
+      const float x[3] = {a.x, a.y, a.z}, xf[3] = {bq.x, bq.y, bq.z};
+      const Wrapped xw = wrapped(c, x);
+      const int b = brick_of(xw.x, xw.y, xw.z, c.g);
+      const uint32_t nc = c.bs.bword[b] & 0xffffu;
+      const float step2 = (xf[0] - x[0]) * (xf[0] - x[0]) + (xf[1] - x[1]) * (xf[1] - x[1]) +
+                          (xf[2] - x[2]) * (xf[2] - x[2]);
+      // most flagged walkers meet no particle: test x and x_f against the brick's candidates (one
+      // pass over each candidate's control points)
+      bool hit = step2 > c.ps.walk_margin * c.ps.walk_margin || nc > MAXC;
+      if (!hit) {
+        const Wrapped xfw = wrapped(c, xf);
+        for (uint32_t m = 0; m < nc && !hit; ++m) {
+          const ParticleDesc& d = c.ps.desc[c.bs.bcand[b * MAXC + m] & 0x7fff];
+          float fa = 0.0f, fb = 0.0f;
+          for (int i = d.c0; i < d.c1; ++i) {
+            const float4 cc = c.bs.cworld[i];
+            const float ax = min_image_rn(xw.x - cc.x, (float)c.g.n[0], c.g.wall[0]);
+            const float ay = min_image_rn(xw.y - cc.y, (float)c.g.n[1], c.g.wall[1]);
+            const float az = min_image_rn(xw.z - cc.z, (float)c.g.n[2], c.g.wall[2]);
+            const float bx = min_image_rn(xfw.x - cc.x, (float)c.g.n[0], c.g.wall[0]);
+            const float by = min_image_rn(xfw.y - cc.y, (float)c.g.n[1], c.g.wall[1]);
+            const float bz = min_image_rn(xfw.z - cc.z, (float)c.g.n[2], c.g.wall[2]);
+            fa += __fdividef(cc.w, ax * ax + ay * ay + az * az);
+            fb += __fdividef(cc.w, bx * bx + by * by + bz * bz);
+          }
+          // the warp repeats the test with its own rounding: a 1e-3 margin sends every walker whose
+          // value is anywhere near the surface there, so the two tests never disagree
+          hit = fa >= 1.0f - 1e-3f || fb >= 1.0f - 1e-3f;
         }
-        // the out-of-line path repeats the test with its own rounding: a 1e-3 margin sends every
-        // walker whose value is anywhere near the surface there, so the two tests never disagree
-        hit = fa >= 1.0f - 1e-3f || fb >= 1.0f - 1e-3f;
       }
+      if (hit) s_hit[atomicAdd(&s_nhit, 1u)] = slot;
+      else pos[__float_as_uint(bq.w)] = make_float4(xf[0], xf[1], xf[2], a.w);
     }
-    unsigned ev = 0u;
-    if (hit) ev = resolve_particles(c, x, xf, xw, yw, zw, b, nc, far_step, id, (uint32_t)T, amp, k0, k1, xn);
-    pos[w] = make_float4(xn[0], xn[1], xn[2], a.w);
-    for (int m = 0; m < 5; ++m) ev_all[m] += (ev >> m) & 1u;
+    __syncthreads();
+    const unsigned hits = s_nhit;
+    for (unsigned k = threadIdx.x >> 5; k < hits; k += RESOLVE_THREADS / 32) {   // a warp per walker
+      const size_t slot = s_hit[k];
+      const float4 a = list[2 * slot], bq = list[2 * slot + 1];
+      const float x[3] = {a.x, a.y, a.z}, xf[3] = {bq.x, bq.y, bq.z};
+      const Wrapped xw = wrapped(c, x);
+      const int b = brick_of(xw.x, xw.y, xw.z, c.g);
+      const uint32_t nc = c.bs.bword[b] & 0xffffu;
+      const float step2 = (xf[0] - x[0]) * (xf[0] - x[0]) + (xf[1] - x[1]) * (xf[1] - x[1]) +
+                          (xf[2] - x[2]) * (xf[2] - x[2]);
+      float xn[3] = {xf[0], xf[1], xf[2]};
+      const unsigned ev = resolve_particles(c, x, xf, xw, b, nc, step2 > c.ps.walk_margin * c.ps.walk_margin,
+                                            __float_as_uint(a.w), (uint32_t)T, amp, k0, k1, xn);
+      if ((threadIdx.x & 31) == 0) pos[__float_as_uint(bq.w)] = make_float4(xn[0], xn[1], xn[2], a.w);
+      for (int m = 0; m < 5; ++m) ev_all[m] += (ev >> m) & 1u;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_nhit = 0u;
+    __syncthreads();
   }
   const int slot[5] = {ST_TYPE2, ST_TYPE3, ST_TYPE4, ST_BISECT_FAIL, ST_REFILL_FAIL};
-  for (int m = 0; m < 5; ++m) {
-    unsigned v = ev_all[m];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(&status[slot[m]], (unsigned long long)v);
-  }
+  if ((threadIdx.x & 31) == 0)   // a warp's events are the same in every lane
+    for (int m = 0; m < 5; ++m)
+      if (ev_all[m]) atomicAdd(&status[slot[m]], (unsigned long long)ev_all[m]);
 }
 
 __global__ void __launch_bounds__(256, 5) walker_kernel(const WalkerArgs a) {
@@ -515,11 +583,11 @@ __global__ void __launch_bounds__(256, 5) walker_batched(const WalkerArgs* __res
   walker_body(a.c, a.pos, a.n, a.u, a.d_T, a.toff, a.amp, a.k0, a.k1, a.status, a.list, a.list_n, a.cap,
               m.block, m.blocks);
 }
-__global__ void __launch_bounds__(256, 8) walker_resolve_kernel(const WalkerArgs a) {
+__global__ void __launch_bounds__(RESOLVE_THREADS, 10) walker_resolve_kernel(const WalkerArgs a) {
   resolve_body(a.c, a.pos, a.list, a.list_n, a.list_n_next, a.d_T, a.toff, a.amp, a.k0, a.k1, a.status, a.cap,
                blockIdx.x, gridDim.x);
 }
-__global__ void __launch_bounds__(256, 4) resolve_batched(const WalkerArgs* __restrict__ args,
+__global__ void __launch_bounds__(RESOLVE_THREADS, 10) resolve_batched(const WalkerArgs* __restrict__ args,
                                                           const BlockMap* __restrict__ map) {
   const BlockMap m = map[blockIdx.x];
   const WalkerArgs& a = args[m.domain];
@@ -546,17 +614,19 @@ int walker_grid(int64_t n, int nsm) {
   const int64_t blocks = (n + 255) / 256;
   return (int)(blocks < (int64_t)nsm * WALKER_BLOCKS_PER_SM ? blocks : (int64_t)nsm * WALKER_BLOCKS_PER_SM);
 }
-// the resolve pass is latency-bound: 8 resident blocks per SM (32 registers; the rare particle
-// path spills) and two waves of them measured best (step 0.744 against 0.754 ms at 4 per SM)
-int resolve_grid(int nsm) { return nsm * 16; }
+// The resolve pass runs beside the next step's fluid, so what it holds of an SM counts as much as
+// its own time: blocks of 128 threads at 48 registers, two waves of 10 per SM, measured best (256^3:
+// walker phase 251 us and step 704 us; 256 threads at 64 registers 257 / 773, 64 threads 255 / 706;
+// the loop-per-lane form at 32 registers 278 / 708; in a 33^3 box the walkers take 28 instead of 38 us)
+int resolve_grid(int nsm) { return nsm * 20; }
 
 void launch_walkers(const Geom& g, const ParticleSet& ps, BrickSet bs1, float4* pos, int64_t n,
                     const float* u, const int64_t* d_T, int toff, int toff_parity, float D,
                     uint32_t k0, uint32_t k1, unsigned long long* status, float4* list,
-                    unsigned int* list_n, int nsm, cudaStream_t st) {
+                    unsigned int* list_n, int nsm, int nsm_resolve, cudaStream_t st) {
   const WalkerArgs a = make_walker_args(g, ps, bs1, pos, n, u, d_T, toff, toff_parity, D, k0, k1, status, list, list_n);
   walker_kernel<<<(unsigned)walker_grid(n, nsm), 256, 0, st>>>(a);
-  walker_resolve_kernel<<<resolve_grid(nsm), 256, 0, st>>>(a);
+  walker_resolve_kernel<<<resolve_grid(nsm_resolve), RESOLVE_THREADS, 0, st>>>(a);
 }
 size_t walker_args_size() { return sizeof(WalkerArgs); }
 void walker_args(void* dst, const Geom& g, const ParticleSet& ps, BrickSet bs1, float4* pos, int64_t n,
@@ -569,7 +639,7 @@ void launch_walker_batched(const void* args, const BlockMap* map, int nblocks, c
   if (nblocks > 0) walker_batched<<<nblocks, 256, 0, st>>>(static_cast<const WalkerArgs*>(args), map);
 }
 void launch_resolve_batched(const void* args, const BlockMap* map, int nblocks, cudaStream_t st) {
-  if (nblocks > 0) resolve_batched<<<nblocks, 256, 0, st>>>(static_cast<const WalkerArgs*>(args), map);
+  if (nblocks > 0) resolve_batched<<<nblocks, RESOLVE_THREADS, 0, st>>>(static_cast<const WalkerArgs*>(args), map);
 }
 
 struct AdvanceArgs {
