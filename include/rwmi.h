@@ -388,7 +388,8 @@ RWMI_API rwmi_status rwmi_batch_set_mode(rwmi_batch* batch, int32_t mode);
 /* Work split of the fused launches (the "tiles"): threads per LBM block (64, 128, 256; one cell
  * per thread), 256-walker chunks per walker block (1..64), walkers per block of the particle-
  * resolution pass (>= 256; at most the single-context grid), bricks per raster block (>= 1).
- * Defaults {128, 1, 8192, 64}. Setting them drops the captured graphs (re-captured at the next
+ * Defaults {128, 1, 8192, 64}. Where the last two would leave SMs empty, a domain gets its share of
+ * a full grid instead. Setting them drops the captured graphs (re-captured at the next
  * step). Results do not depend on them. */
 typedef struct {
   int32_t lbm_block;
