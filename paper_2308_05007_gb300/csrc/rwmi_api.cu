@@ -64,6 +64,7 @@ struct rwmi_ctx {
   cudaStream_t side = nullptr;    // raster of t+1 beside the LBM of t
   cudaStream_t wst = nullptr;     // walkers of t beside the fluid of t+1
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr, fluid_ev = nullptr, walk_ev[2] = {nullptr, nullptr};
+  cudaEvent_t start_ev = nullptr;   // every block of the resolve pass has begun
   bool stepped = false;
   std::string err;
 
@@ -123,6 +124,7 @@ struct rwmi_ctx {
   int64_t t = 0;
   int64_t t_base = 0;   // value of the device counter d_T: t at the start of the current run
   bool walk_rec[2] = {false, false};   // walk_ev[p] recorded in the current run
+  bool start_rec = false;              // start_ev likewise
   int fcur = 0, pcur = 0;
   int64_t binned_t = -1;
   int64_t series_rows = 0;
@@ -611,6 +613,12 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     // present resolve pass). The walkers stay on their own stream: queued in this one, before the
     // clear or behind the poses, runs at 256^3 took 2.5 to 7% longer.
     pose();
+    // behind a pass 1 that filled every SM, the raster and the update wait until the resolve pass's
+    // blocks have begun: it is the chain the next step's walkers wait for, and on some GPUs the
+    // update's blocks took the SMs before it (256^3 run of 32 steps on such a GPU: 24.6 ms, 23.2 ms
+    // with the wait before the raster, 24.8 ms with it before the clear). A pass 1 that leaves
+    // SMs free leaves room for the resolve pass too, so small runs take no extra dependency.
+    if (c->start_rec) cudaStreamWaitEvent(c->stream, c->start_ev, 0);
     launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, part, c->stream);
     c->launches++;
     lbm(true);
@@ -640,8 +648,10 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
   }
   phase_begin(c, RWMI_PHASE_WALKERS);
   if (c->nw > 0) {
+    const bool ordered = ws != c->stream && fork_raster && !ibb && !dem && walkers_fill_chip(c->nw, c->nsm);
     launch_walkers(c->g, ps, brick_set(c, tn), c->pos[c->pcur], c->nw, c->u[tp], c->d_T, toff, tp, (float)c->D,
-                   k0, k1, c->status, c->wlist, c->wlist_n, c->nsm, part, ws);
+                   k0, k1, c->status, c->wlist, c->wlist_n, c->nsm, part, ws, ordered ? c->start_ev : nullptr);
+    c->start_rec = ordered;
     c->launches += 2;
   }
   phase_end(c, RWMI_PHASE_WALKERS);
@@ -672,6 +682,7 @@ void segment_end(rwmi_ctx* c) {
   if (c->walk_rec[0] || c->walk_rec[1]) {
     cudaStreamWaitEvent(c->stream, c->walk_ev[(c->t - 1) & 1], 0);
     c->walk_rec[0] = c->walk_rec[1] = false;
+    c->start_rec = false;
   }
   if (c->t > c->t_base) {
     launch_advance(c->d_T, c->t - c->t_base, c->stream);
@@ -774,7 +785,7 @@ RWMI_API rwmi_status rwmi_create(rwmi_ctx** out, const int32_t dims[3], double t
       for (int k = 0; k < 2; ++k) CK(dalloc(c, &c->node[k], sizeof(uint16_t) * (size_t)ncell));
       CK(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
       CK(cudaStreamCreateWithFlags(&c->wst, cudaStreamNonBlocking));
-      for (cudaEvent_t* e : {&c->fork_ev, &c->join_ev, &c->fluid_ev, &c->walk_ev[0], &c->walk_ev[1]})
+      for (cudaEvent_t* e : {&c->fork_ev, &c->join_ev, &c->fluid_ev, &c->walk_ev[0], &c->walk_ev[1], &c->start_ev})
         CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
       CK(dalloc(c, &c->d_T, sizeof(int64_t)));
       CK(dalloc(c, &c->wlist_n, sizeof(unsigned int) * 2 * WLIST_STRIPES));
@@ -2269,7 +2280,7 @@ RWMI_API void rwmi_destroy(rwmi_ctx* c) {
   cudaStreamSynchronize(c->stream);   // the frees have returned the memory when this returns
   for (int k = 0; k < 2 * RWMI_NPHASE; ++k)
     if (c->ev[k]) cudaEventDestroy(c->ev[k]);
-  for (cudaEvent_t e : {c->fork_ev, c->join_ev, c->fluid_ev, c->walk_ev[0], c->walk_ev[1]})
+  for (cudaEvent_t e : {c->fork_ev, c->join_ev, c->fluid_ev, c->walk_ev[0], c->walk_ev[1], c->start_ev})
     if (e) cudaEventDestroy(e);
   if (c->side) cudaStreamDestroy(c->side);
   if (c->wst) cudaStreamDestroy(c->wst);

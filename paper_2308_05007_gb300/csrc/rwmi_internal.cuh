@@ -345,10 +345,12 @@ inline int64_t wlist_stripe_cap(int64_t n) {
 }
 // list_n: 2 * WLIST_STRIPES counters, one set per time parity (toff_parity = t mod 2); both
 // sets must be zero before the first step.
+bool walkers_fill_chip(int64_t n, int nsm);   // pass 1's grid takes its full share of every SM
+// started: recorded once every block of the resolve pass has begun (nullptr: not recorded).
 void launch_walkers(const Geom& g, const ParticleSet& ps, BrickSet bs1, float4* pos, int64_t n,
                     const float* u, const int64_t* d_T, int toff, int toff_parity, float D,
                     uint32_t k0, uint32_t k1, unsigned long long* status, float4* list,
-                    unsigned int* list_n, int nsm, int nsm_resolve, cudaStream_t st);
+                    unsigned int* list_n, int nsm, int nsm_resolve, cudaStream_t st, cudaEvent_t started);
 void launch_advance(int64_t* d_T, int64_t k, cudaStream_t st);
 void launch_seed(const Geom& g, const ParticleSet& ps, BrickSet bs, float4* pos, float4* x0,
                  int64_t n, const double lo[3], const double hi[3], uint32_t k0, uint32_t k1,

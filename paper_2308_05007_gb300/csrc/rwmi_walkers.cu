@@ -620,13 +620,25 @@ int walker_grid(int64_t n, int nsm) {
 // the loop-per-lane form at 32 registers 278 / 708; in a 33^3 box the walkers take 28 instead of 38 us)
 int resolve_grid(int nsm) { return nsm * 20; }
 
+bool walkers_fill_chip(int64_t n, int nsm) { return walker_grid(n, nsm) == nsm * WALKER_BLOCKS_PER_SM; }
+
 void launch_walkers(const Geom& g, const ParticleSet& ps, BrickSet bs1, float4* pos, int64_t n,
                     const float* u, const int64_t* d_T, int toff, int toff_parity, float D,
                     uint32_t k0, uint32_t k1, unsigned long long* status, float4* list,
-                    unsigned int* list_n, int nsm, int nsm_resolve, cudaStream_t st) {
+                    unsigned int* list_n, int nsm, int nsm_resolve, cudaStream_t st, cudaEvent_t started) {
   const WalkerArgs a = make_walker_args(g, ps, bs1, pos, n, u, d_T, toff, toff_parity, D, k0, k1, status, list, list_n);
   walker_kernel<<<(unsigned)walker_grid(n, nsm), 256, 0, st>>>(a);
-  walker_resolve_kernel<<<resolve_grid(nsm_resolve), RESOLVE_THREADS, 0, st>>>(a);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)resolve_grid(nsm_resolve));
+  cfg.blockDim = dim3(RESOLVE_THREADS);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeLaunchCompletionEvent;
+  at[0].val.launchCompletionEvent.event = started;
+  at[0].val.launchCompletionEvent.flags = 0;
+  cfg.attrs = at;
+  cfg.numAttrs = started ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, walker_resolve_kernel, a);
 }
 size_t walker_args_size() { return sizeof(WalkerArgs); }
 void walker_args(void* dst, const Geom& g, const ParticleSet& ps, BrickSet bs1, float4* pos, int64_t n,
