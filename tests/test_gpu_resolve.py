@@ -64,3 +64,26 @@ def test_walkers_at_surfaces_match_the_oracle(name):
             xo = ora.walkers_advance(x_prev.astype(np.float64), np.arange(len(x_prev), dtype=np.uint32))
             d = np.abs(x_next - xo).max(1)
             assert (d > 2e-5).mean() <= 1e-3, np.sort(d)[-5:]
+
+
+@pytest.mark.parametrize("blocks", [-1, 0, 3])
+def test_raster_waits_for_resolve_pass(blocks):
+    """Walkers that leave pass 1's resident grid (5 blocks of 256 per SM) one block short, fill it, or
+    loop in it: the raster's wait for the resolve pass changes no bit against one stream, in
+    captured and in eager runs of several steps."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2308_05007_gb300.rwmi import Simulation
+    n = 256 * (5 * torch.cuda.get_device_properties(0).multi_processor_count + blocks) - 7
+    dims, walls, particles = CASES["remainder"]
+    w = I.Workload(name="grid", dims=dims, tau=0.8, D=0.01, seed=7, wall_mask=walls, n_walkers=n,
+                   walker_box=((0.0, 0.0, 0.0), tuple(float(v) for v in dims)), metaballs=_metaballs(particles))
+    runs = []
+    for overlap, graphs in ((0, 1), (2, 1), (2, 0)):
+        with Simulation.from_workload(w, overlap=overlap, use_graphs=graphs) as sim:
+            for k in (9, 16, 5):
+                sim.step(k)
+            runs.append((sim.walkers_by_id()[0], sim.velocity(), sim.solid()[0]))
+    for other in runs[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(runs[0], other))
