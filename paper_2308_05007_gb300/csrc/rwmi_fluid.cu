@@ -164,33 +164,13 @@ __device__ void pose_bin_body(const PoseArgs& A, int blk, int nblk) {
   // particle within the walker margin
   const float Rw = d.rb + ps.walk_margin;
   if (warp == 7) {
-    // Per axis (one lane each), the bricks met by the interval [o - Rw, o + Rw] of the wrapped
-    // domain: one range, or two when the interval crosses a periodic face (bricks need not tile a
-    // periodic axis evenly, so the wrap is done on cell coordinates, not brick indices).
+    // per axis (one lane each), the bricks met by the interval [o - Rw, o + Rw]
     if (lane < 3) {
       const int a = lane;
-      const double n = (double)g.n[a], lo = s_ow[a] - Rw, hi = s_ow[a] + Rw;
-      const int last = g.nb[a] - 1;
-      int nr = 1, a0 = 0, b0 = last, a1 = 0, b1 = 0;
-      if (g.wall[a]) {
-        const double l = fmax(lo, 0.0), h = fmin(hi, n);
-        nr = l <= h ? 1 : 0;
-        a0 = min((int)floor(l / BRICK), last);
-        b0 = min((int)floor(h / BRICK), last);
-      } else if (hi - lo < n) {
-        const double s0 = lo - n * floor(lo / n), e0 = s0 + (hi - lo);
-        a0 = min((int)floor(s0 / BRICK), last);
-        if (e0 < n) {
-          b0 = min((int)floor(e0 / BRICK), last);
-        } else {
-          b1 = min((int)floor((e0 - n) / BRICK), last);
-          if (b1 >= a0 - 1) a0 = 0;
-          else nr = 2;
-        }
-      }
-      s_ra[a][0] = a0; s_rb[a][0] = b0;
-      s_ra[a][1] = a1; s_rb[a][1] = b1;
-      s_nr[a] = nr;
+      const BrickRange r = brick_range(s_ow[a], Rw, g.n[a], g.nb[a], g.wall[a]);
+      s_ra[a][0] = r.a[0]; s_rb[a][0] = r.b[0];
+      s_ra[a][1] = r.a[1]; s_rb[a][1] = r.b[1];
+      s_nr[a] = r.n;
     }
   } else {   // world control points, one coordinate per lane of warps 0-6
     for (int k = threadIdx.x; k < 3 * (d.c1 - d.c0); k += blockDim.x - 32) {

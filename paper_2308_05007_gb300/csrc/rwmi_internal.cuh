@@ -110,6 +110,38 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t v, uint32_t m, uint32_t s)
   return (__umulhi(v, m) + v) >> s;
 }
 
+// Bricks of one axis that the interval [o - R, o + R] meets: n ranges a .. b, two where it crosses a
+// periodic face (bricks need not tile a periodic axis evenly, so the wrap is done on cell
+// coordinates, not brick indices). Whatever o and R are, every range lies within the axis and has
+// a <= b: these are indexes into the brick arrays, and for origins beyond ~1e32 the wrapped
+// coordinate is no longer within the box.
+struct BrickRange { int n, a[2], b[2]; };
+__host__ __device__ inline int brick_of_cell(double x, int nb) {
+  const double f = floor(x / BRICK);
+  return f > 0.0 ? (f < (double)nb ? (int)f : nb - 1) : 0;   // not a number: 0
+}
+__host__ __device__ inline BrickRange brick_range(double o, double R, int cells, int nb, int wall) {
+  const double n = (double)cells, lo = o - R, hi = o + R;
+  BrickRange r{1, {0, 0}, {nb - 1, 0}};
+  if (wall) {
+    const double l = fmax(lo, 0.0), h = fmin(hi, n);
+    r.a[0] = brick_of_cell(l, nb);
+    r.b[0] = brick_of_cell(h, nb);
+    if (!(l <= h)) r = BrickRange{0, {0, 0}, {0, 0}};
+  } else if (hi - lo < n) {
+    const double s0 = lo - n * floor(lo / n), e0 = s0 + (hi - lo);
+    r.a[0] = brick_of_cell(s0, nb);
+    if (e0 < n) {
+      r.b[0] = brick_of_cell(e0, nb);
+    } else {
+      r.b[1] = brick_of_cell(e0 - n, nb);
+      if (r.b[1] >= r.a[0] - 1) r.a[0] = 0;
+      else r.n = 2;
+    }
+  }
+  return r;
+}
+
 // ---- Philox4x32-10 (Salmon et al., SC'11): ten rounds of two 32x32->64 products ----
 __device__ __forceinline__ uint4 philox(uint4 c, uint32_t k0, uint32_t k1) {
 #pragma unroll
