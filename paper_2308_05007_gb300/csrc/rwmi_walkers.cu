@@ -184,9 +184,10 @@ __device__ __forceinline__ bool beyond_bound(const WalkCtx& c, int p, const Wrap
   return dx * dx + dy * dy + dz * dz > rb * rb;
 }
 
-// Lowest-index particle holding x, or -1, through the candidate list of x's own brick: a particle
-// holding x lies within its bound radius of x, so it is on that list (built at the same time with a
-// larger radius); all particles when the list overflowed.
+// Lowest-index particle holding x, or -1, by one warp: a lane per candidate of x's own brick for the
+// bound radius, then Eq. 3 of those within it. A particle holding x lies within its bound radius of x, so
+// it is on that list (built at the same time with a larger radius); all particles when the list
+// overflowed.
 __device__ int inside_cand(const WalkCtx& c, WarpParticle& h, const float* x) {
   const Wrapped w = wrapped(c, x);
   const int b = brick_of(w.x, w.y, w.z, c.g);
@@ -194,12 +195,16 @@ __device__ int inside_cand(const WalkCtx& c, WarpParticle& h, const float* x) {
   const bool all = nc > MAXC;
   const uint32_t n = all ? (uint32_t)c.ps.P : nc;
   int best = -1;
-  for (uint32_t m = 0; m < n; ++m) {
-    const int p = all ? (int)m : (c.bs.bcand[b * MAXC + m] & 0x7fff);
-    if (best >= 0 && p > best) continue;
-    if (beyond_bound(c, p, w)) continue;
-    hold(c, p, h);
-    if (warp_value(c, h, w) >= 1.0f) best = p;
+  for (uint32_t base = 0; base < n; base += 32) {
+    const uint32_t m = base + (threadIdx.x & 31);
+    const int mine = m >= n ? -1 : all ? (int)m : (c.bs.bcand[b * MAXC + m] & 0x7fff);
+    unsigned near = __ballot_sync(0xffffffffu, mine >= 0 && !beyond_bound(c, mine, w));
+    for (; near; near &= near - 1u) {
+      const int p = __shfl_sync(0xffffffffu, mine, __ffs(near) - 1);
+      if (best >= 0 && p > best) continue;
+      hold(c, p, h);
+      if (warp_value(c, h, w) >= 1.0f) best = p;
+    }
   }
   return best;
 }
@@ -255,18 +260,25 @@ __device__ bool refill(const WalkCtx& c, WarpParticle& h, int p, const float* x,
   sincospif(2.0f * uniform24(r.y), &sp, &cp);
   const float rad = amp * cbrtf(uniform24(r.z));
   float xr[3] = {xs[0] + rad * st * cp, xs[1] + rad * st * sp, xs[2] + rad * ct};
-  wall_reflect(xr, c.g);
-  if (inside_cand(c, h, xr) >= 0) {
+  // the drawn point, its mirror image in the surface's tangent plane, the outside end of the bisection:
+  // the first that no particle holds. Loops here and at the two points of a long step keep one copy of
+  // the test: the pass ends with a few walkers, whose time is that of fetching their code (96^3,
+  // walkers 79 -> 75 us).
+#pragma unroll 1
+  for (int k = 0; k < 3; ++k) {
+    if (k < 2) wall_reflect(xr, c.g);
+    const bool held = inside_cand(c, h, xr) >= 0;
+    if (!held || k == 2) {
+      xnew[0] = xr[0]; xnew[1] = xr[1]; xnew[2] = xr[2];
+      return !held;
+    }
     const float dn = (xr[0] - xs[0]) * no[0] + (xr[1] - xs[1]) * no[1] + (xr[2] - xs[2]) * no[2];
-    if (dn < 0.0f) for (int a = 0; a < 3; ++a) xr[a] -= 2.0f * dn * no[a];
-    wall_reflect(xr, c.g);
-    if (inside_cand(c, h, xr) >= 0) {
-      xr[0] = aend[0]; xr[1] = aend[1]; xr[2] = aend[2];
-      if (inside_cand(c, h, xr) >= 0) { xnew[0] = xr[0]; xnew[1] = xr[1]; xnew[2] = xr[2]; return false; }
+    for (int a = 0; a < 3; ++a) {
+      if (k == 1) xr[a] = aend[a];
+      else if (dn < 0.0f) xr[a] -= 2.0f * dn * no[a];
     }
   }
-  xnew[0] = xr[0]; xnew[1] = xr[1]; xnew[2] = xr[2];
-  return true;
+  return false;
 }
 
 // Types II-IV of one walker (x to x_f) against the particles at t+1: candidates of the walker's brick
@@ -280,8 +292,12 @@ __device__ unsigned resolve_particles(const WalkCtx& c, const float* x, const fl
   WarpParticle h;
   h.p = -1;
   if (nc > MAXC || far_step) {
-    pin = inside_cand(c, h, x);
-    qin = inside_cand(c, h, xf);
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+      const float at[3] = {k ? xf[0] : x[0], k ? xf[1] : x[1], k ? xf[2] : x[2]};
+      const int in = inside_cand(c, h, at);
+      if (k) qin = in; else pin = in;
+    }
   } else {
     const Wrapped xfw = wrapped(c, xf);
     for (uint32_t m = 0; m < nc; ++m) {
@@ -518,13 +534,23 @@ __device__ __forceinline__ void resolve_body(const WalkCtx& c, float4* __restric
       const uint32_t nc = c.bs.bword[b] & 0xffffu;
       const float step2 = (xf[0] - x[0]) * (xf[0] - x[0]) + (xf[1] - x[1]) * (xf[1] - x[1]) +
                           (xf[2] - x[2]) * (xf[2] - x[2]);
-      // most flagged walkers meet no particle: test x and x_f against the brick's candidates (one
-      // pass over each candidate's control points)
-      bool hit = step2 > c.ps.walk_margin * c.ps.walk_margin || nc > MAXC;
-      if (!hit) {
-        const Wrapped xfw = wrapped(c, xf);
-        for (uint32_t m = 0; m < nc && !hit; ++m) {
-          const ParticleDesc& d = c.ps.desc[c.bs.bcand[b * MAXC + m] & 0x7fff];
+      // most flagged walkers meet no particle: test x and x_f against the candidates of x's brick in one
+      // pass over each one's control points, after an unusually long step against those of x_f's brick
+      // as well; against every particle where a list overflowed. Crowded bricks and fast streams send
+      // all their walkers here: with a warp for each, untested, the walkers of a 48^3 box of 343
+      // spheres (1e6 walkers) took 8.2 ms, those of a 96^3 stream at 0.2 414 us; now 530 and 92 us.
+      const Wrapped xfw = wrapped(c, xf);
+      int at = b;
+      uint32_t n = nc;
+      bool hit = false, last = !(step2 > c.ps.walk_margin * c.ps.walk_margin);
+#pragma unroll 1
+      for (;;) {
+        const bool all = n > MAXC;
+        if (all) n = (uint32_t)c.ps.P;
+        for (uint32_t m = 0; m < n && !hit; ++m) {
+          const int p = all ? (int)m : (c.bs.bcand[at * MAXC + m] & 0x7fff);
+          if (all && beyond_bound(c, p, xw) && beyond_bound(c, p, xfw)) continue;
+          const ParticleDesc& d = c.ps.desc[p];
           float fa = 0.0f, fb = 0.0f;
           for (int i = d.c0; i < d.c1; ++i) {
             const float4 cc = c.bs.cworld[i];
@@ -541,6 +567,10 @@ __device__ __forceinline__ void resolve_body(const WalkCtx& c, float4* __restric
           // value is anywhere near the surface there, so the two tests never disagree
           hit = fa >= 1.0f - 1e-3f || fb >= 1.0f - 1e-3f;
         }
+        if (last || hit || all) break;
+        last = true;
+        at = brick_of(xfw.x, xfw.y, xfw.z, c.g);
+        n = c.bs.bword[at] & 0xffffu;
       }
       if (hit) s_hit[atomicAdd(&s_nhit, 1u)] = slot;
       else pos[__float_as_uint(bq.w)] = make_float4(xf[0], xf[1], xf[2], a.w);
