@@ -502,22 +502,22 @@ struct RasterArgs {
   uint16_t* nodes;
 };
 
-__device__ __forceinline__ void raster_body(const RasterArgs& A, int blk, int nblk) {
+// CLASSES: node classes instead of counts. WHOLE: a list that keeps whole bricks (plog = 0); the
+// arithmetic of slices and parts then falls away.
+template <bool CLASSES, bool WHOLE>
+__device__ __forceinline__ void raster_list(const RasterArgs& A, RasterWarp* s_rw, int blk, uint32_t warps,
+                                            uint32_t nlist, int plog) {
   const Geom g = A.g;
   const ParticleSet ps = A.ps;
   const BrickSet bs = A.bs;
-  const bool classes = A.nodes != nullptr;
-  uint16_t* __restrict__ solid = classes ? A.nodes : A.solid;   // the words of cells written
+  uint16_t* __restrict__ solid = CLASSES ? A.nodes : A.solid;   // the words of cells written
   unsigned long long* __restrict__ status = A.status;
-  __shared__ RasterWarp s_rw[RW_WARPS];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   RasterWarp& W = s_rw[wib];
   const uint32_t nbrick = (uint32_t)g.nb[0] * g.nb[1] * g.nb[2];
-  const uint32_t nlist = bs.bword[nbrick];
-  const uint32_t warps = (uint32_t)nblk * RW_WARPS;
-  // node classes are a few rounds per brick: whole bricks there
-  const int plog = classes ? 0 : raster_pieces_log2(nlist, warps), slog = min(plog, 3), parts = 1 << (plog - slog);
+  if (WHOLE) plog = 0;
+  const int slog = min(plog, 3), parts = 1 << (plog - slog);
   const uint32_t units = nlist << plog;
   const int K = 64 >> slog;          // mini-bricks per slice: 64, 32, 16 or 8
   const int rows_y = K >= 16 ? 8 : 4;   // cell rows of a slice along y
@@ -618,7 +618,7 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A, int blk, int nb
           listed = listed && bi * BRICK + 2 * (mb & 3) < g.n[0] && bj * BRICK + 2 * ((mb >> 2) & 3) < g.n[1] &&
                    bk * BRICK + 2 * (mb >> 4) < g.n[2];
           W.val[mb] = listed ? (uint16_t)RW_LISTED : own == 0x7fffffff ? (uint16_t)0
-                      : classes               ? (uint16_t)(1 + own)
+                      : CLASSES               ? (uint16_t)(1 + own)
                                               : (uint16_t)(64 | (own << 7));
         }
         wm[h] = __ballot_sync(full, need);
@@ -670,7 +670,7 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A, int blk, int nb
       const int i = bi * BRICK + lx, j = bj * BRICK + ly, k = bk * BRICK + lz;
       const bool in_dom = have && i < g.n[0] && j < g.n[1] && k < g.n[2];
       const float xi = (float)i, yj = (float)j, zk = (float)k;
-      if (classes) {
+      if (CLASSES) {
         const float xs = xi + 0.5f, ys = yj + 0.5f, zs = zk + 0.5f;
         int own = 0x7fffffff;
         for (int m = 0; in_dom && m < (staged ? n : over ? ps.P : (int)nc); ++m) {
@@ -761,15 +761,32 @@ __device__ __forceinline__ void raster_body(const RasterArgs& A, int blk, int nb
   if (lane == 0 && queued) atomicAdd(&status[ST_RASTER_QUEUED], queued);
 }
 
+__device__ __forceinline__ uint32_t raster_list_length(const RasterArgs& A) {
+  return A.bs.bword[(uint32_t)A.g.nb[0] * A.g.nb[1] * A.g.nb[2]];
+}
+
+// Three forms, each compiled by itself: run-time slices and the class switch inside one body cost every
+// brick of a long list (256^3, 13 k bricks: 209 us, 183 apart; 384^3, 27 k: 377 and 317 us). The pieces'
+// form comes first in the code: behind the other it took 10 to 15% longer (96^3 and below).
+template <bool CLASSES>
 __global__ void __launch_bounds__(256, 4) raster_kernel(const RasterArgs a) {
   asm volatile("griddepcontrol.launch_dependents;");   // the LBM update may fill the rest of each SM now
-  raster_body(a, blockIdx.x, gridDim.x);
+  __shared__ RasterWarp s_rw[RW_WARPS];
+  const uint32_t nlist = raster_list_length(a), warps = gridDim.x * RW_WARPS;
+  const int plog = CLASSES ? 0 : raster_pieces_log2(nlist, warps);   // node classes are a few rounds per brick
+  if (!CLASSES && plog > 0) raster_list<CLASSES, false>(a, s_rw, blockIdx.x, warps, nlist, plog);
+  else raster_list<CLASSES, true>(a, s_rw, blockIdx.x, warps, nlist, 0);
 }
-__global__ void __launch_bounds__(256, 4) raster_batched(const RasterArgs* __restrict__ args,
+// The pieces' form for every domain (small ones, whose lists are short), with more registers, since
+// the arguments come from memory rather than the constant bank.
+__global__ void __launch_bounds__(256, 3) raster_batched(const RasterArgs* __restrict__ args,
                                                          const BlockMap* __restrict__ map) {
   asm volatile("griddepcontrol.launch_dependents;");   // as raster_kernel
+  __shared__ RasterWarp s_rw[RW_WARPS];
   const BlockMap m = map[blockIdx.x];
-  raster_body(args[m.domain], m.block, m.blocks);
+  const RasterArgs& A = args[m.domain];
+  const uint32_t nlist = raster_list_length(A), warps = (uint32_t)m.blocks * RW_WARPS;
+  raster_list<false, false>(A, s_rw, m.block, warps, nlist, raster_pieces_log2(nlist, warps));
 }
 
 // two blocks per SM: the raster runs beside the LBM, which takes the rest of each SM (four
@@ -779,7 +796,9 @@ int raster_grid(int nsm) { return nsm * 2; }
 void launch_raster(const Geom& g, const ParticleSet& ps, BrickSet bs, uint16_t* solid,
                    unsigned long long* status, int nsm, cudaStream_t st, uint16_t* nodes) {
   if (ps.P == 0) return;
-  raster_kernel<<<raster_grid(nsm), RW_WARPS * 32, 0, st>>>(RasterArgs{g, ps, bs, solid, status, nodes});
+  const RasterArgs a{g, ps, bs, solid, status, nodes};
+  if (nodes) raster_kernel<true><<<raster_grid(nsm), RW_WARPS * 32, 0, st>>>(a);
+  else raster_kernel<false><<<raster_grid(nsm), RW_WARPS * 32, 0, st>>>(a);
 }
 size_t raster_args_size() { return sizeof(RasterArgs); }
 void raster_args(void* dst, const Geom& g, const ParticleSet& ps, BrickSet bs, uint16_t* solid,
