@@ -1812,7 +1812,11 @@ rwmi_status fused_build_maps(rwmi_batch* b) {
   };
   // The tiles say how much work a block takes at most; where that leaves SMs empty (a few small
   // domains), a domain's raster and resolve passes take their share of a full grid instead: their
-  // bricks and walkers then go to more warps (64 domains of 16^3-48^3: see the raster's pieces).
+  // bricks and walkers then go to more warps (64 domains of 16^3-48^3: see the raster's pieces). For
+  // small domains the raster's full grid is four blocks per SM, as many as fit (64 of 16^3-48^3 277 us
+  // per step, 288 us with two); large ones leave half of each SM to the update, which is the longer
+  // of the two (two of 128^3-160^3 255 us, 262 us with four).
+  const int64_t raster_full = (fused_pays(b) ? 2 : 1) * (int64_t)raster_grid(b->ctxs[0]->nsm);
   int64_t bricks = 1, walkers = 1;
   for (const rwmi_ctx* c : b->ctxs) {
     bricks += c->P > 0 ? c->nbrick : 0;
@@ -1822,7 +1826,7 @@ rwmi_status fused_build_maps(rwmi_batch* b) {
   add(FP_CLEARB, [&](rwmi_ctx* c) { return clear_grid(c->nbrick + BWORD_EXTRA); });
   add(FP_POSE, [&](rwmi_ctx* c) { return c->P > 0 ? c->P : 1; });
   add(FP_RASTER, [&](rwmi_ctx* c) {
-    const int64_t share = 2 * raster_grid(c->nsm) * (int64_t)c->nbrick / bricks;   // four blocks fit an SM
+    const int64_t share = raster_full * (int64_t)c->nbrick / bricks;
     return c->P > 0 ? std::min<int64_t>(std::max<int64_t>({ceil_div(c->nbrick, tl.raster_bricks_per_block), share, 1}),
                                         raster_grid(c->nsm))
                     : 0;
