@@ -255,6 +255,13 @@ RWMI_API rwmi_status rwmi_step_timed(rwmi_ctx* ctx, int32_t n, double* phase_ms)
  * tuner: small or oddly shaped boxes favour smaller blocks. */
 RWMI_API rwmi_status rwmi_autotune(rwmi_ctx* ctx, int32_t* chosen);
 
+/* Tells a context that `contexts` contexts (itself among them) step at the same time, so that the
+ * grids of its raster and particle-resolution passes take its part of the GPU: full grids for each
+ * only add work then (bricks cut into more pieces, more blocks to place). Default 1. Asynchronous
+ * and cheap, so it may be called before every rwmi_step with the current count; results do not
+ * depend on it. In a batch the batch's own count holds. RWMI_E_INVALID for contexts < 1. */
+RWMI_API rwmi_status rwmi_set_concurrency(rwmi_ctx* ctx, int32_t contexts);
+
 /* Non-blocking: RWMI_BUSY while GPU work of the context is in flight, RWMI_OK when it is idle. */
 RWMI_API rwmi_status rwmi_query(rwmi_ctx* ctx);
 

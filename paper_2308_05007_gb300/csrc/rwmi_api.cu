@@ -29,16 +29,18 @@ constexpr uint64_t CKPT_DEM_MAGIC = 0x314d4544ULL;  // "DEM1": the free-DEM sect
 // A captured run of steps is fixed by the buffer parities it starts from, its start time modulo
 // the chunk (which steps sort and form moments) and its length.
 struct GraphKey {
-  int fcur, pcur;
+  int fcur, pcur, part;
   int64_t phase, len;
   bool operator<(const GraphKey& o) const {
     if (fcur != o.fcur) return fcur < o.fcur;
     if (pcur != o.pcur) return pcur < o.pcur;
+    if (part != o.part) return part < o.part;
     if (phase != o.phase) return phase < o.phase;
     return len < o.len;
   }
 };
 constexpr int64_t SEGMENT_MAX = 64;    // longest captured run of steps
+constexpr int PART_MIN = 8;             // SMs a context's raster and resolve grids are sized for at least
 constexpr size_t GRAPH_CACHE_MAX = 32;  // captured runs kept per context; beyond, runs are eager
 
 struct GraphEntry {
@@ -58,7 +60,7 @@ struct rwmi_ctx {
   Geom g;
   int device = 0, nsm = 152;
   int nsm_part = 0;   // SMs this context's raster and resolve grids are sized for: all (0), or its part
-                      // when many contexts step concurrently (branches of a batch)
+                      // when many contexts step concurrently (rwmi_set_concurrency, branches of a batch)
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   cudaStream_t side = nullptr;    // raster of t+1 beside the LBM of t
@@ -1188,7 +1190,7 @@ RWMI_API rwmi_status rwmi_step(rwmi_ctx* c, int32_t n) try {
   while (n > 0) {
     const int64_t k = std::min<int64_t>(n, graphs ? G - c->t % L : n);
     n -= (int32_t)k;
-    const GraphKey key{c->fcur, c->pcur, c->t % L, k};
+    const GraphKey key{c->fcur, c->pcur, c->nsm_part, c->t % L, k};
     auto it = graphs ? c->graphs.find(key) : c->graphs.end();
     if (graphs && it != c->graphs.end()) {
       CK(cudaGraphLaunch(it->second.exec, c->stream));
@@ -1306,6 +1308,20 @@ RWMI_API rwmi_status rwmi_autotune(rwmi_ctx* c, int32_t* chosen) try {
   return RWMI_OK;
 } catch (const std::exception& e_) {
   return api_exception(c, "rwmi_autotune", e_);
+}
+
+// The part is taken for the next power of two, so that a count that changes a little from call to
+// call keeps its captured graphs.
+RWMI_API rwmi_status rwmi_set_concurrency(rwmi_ctx* c, int32_t contexts) try {
+  if (!c) return RWMI_E_INVALID;
+  GUARD(c);
+  if (contexts < 1) return fail(c, RWMI_E_INVALID, "rwmi_set_concurrency: at least one context");
+  int n = 1;
+  while (n < contexts && n < c->nsm) n *= 2;
+  c->nsm_part = n > 1 ? std::max(PART_MIN, c->nsm / n) : 0;
+  return RWMI_OK;
+} catch (const std::exception& e_) {
+  return api_exception(c, "rwmi_set_concurrency", e_);
 }
 
 RWMI_API rwmi_status rwmi_query(rwmi_ctx* c) try {
@@ -2091,9 +2107,10 @@ RWMI_API rwmi_status rwmi_batch_step(rwmi_batch* b, int32_t nsteps) try {
         cudaStreamWaitEvent(c->stream, b->fork, 0);
         // Grids that fill the chip for one context only add work for many at a time (a raster cut into
         // more pieces; 24 domains of 48^3-120^3: 1370 us per step, 1080 us with a part each).
-        c->nsm_part = std::max(8, c->nsm / (int)b->ctxs.size());
+        const int own = c->nsm_part;
+        c->nsm_part = std::max(PART_MIN, c->nsm / (int)b->ctxs.size());
         for (int64_t st = 0; st < b->L; ++st) enqueue_step(c, st == b->L - 1);
-        c->nsm_part = 0;
+        c->nsm_part = own;
         segment_end(c);
         cudaEventRecord(b->join[k], c->stream);
         cudaStreamWaitEvent(b->origin, b->join[k], 0);

@@ -22,7 +22,7 @@ STORE_FP32, STORE_FP32_SHIFT, STORE_FP16_SHIFT, STORE_FP64_SHIFT = 0, 1, 2, 3
 
 EXPORTED = ["rwmi_config_defaults", "rwmi_create", "rwmi_configure", "rwmi_set_stream",
             "rwmi_set_metaballs", "rwmi_seed_walkers", "rwmi_set_walkers", "rwmi_step", "rwmi_step_timed",
-            "rwmi_autotune", "rwmi_query", "rwmi_footprint", "rwmi_sync",
+            "rwmi_autotune", "rwmi_set_concurrency", "rwmi_query", "rwmi_footprint", "rwmi_sync",
             "rwmi_time", "rwmi_info", "rwmi_concentration", "rwmi_walker_moments", "rwmi_moment_series",
             "rwmi_velocity", "rwmi_density", "rwmi_populations", "rwmi_lattice", "rwmi_solid", "rwmi_nodes",
             "rwmi_mass_momentum", "rwmi_particle_forces", "rwmi_force_series", "rwmi_walkers", "rwmi_counters",
@@ -111,6 +111,7 @@ def load(build_if_missing: bool = False):
     L.rwmi_step.argtypes = [P, C.c_int32]
     L.rwmi_step_timed.argtypes = [P, C.c_int32, vp]
     L.rwmi_autotune.argtypes = [P, C.POINTER(C.c_int32)]
+    L.rwmi_set_concurrency.argtypes = [P, C.c_int32]
     L.rwmi_query.argtypes = [P]
     L.rwmi_footprint.argtypes = [C.POINTER(C.c_int32), C.c_int32, C.c_int32, C.c_int64, C.c_int32, C.c_int32,
                                  C.POINTER(C.c_uint64)]
@@ -425,6 +426,10 @@ class Simulation:
         v = C.c_int32()
         self._check(self._L.rwmi_autotune(self._h, C.byref(v)))
         return int(v.value)
+
+    def set_concurrency(self, contexts: int):
+        """Contexts stepping at the same time, this one among them (rwmi_set_concurrency)."""
+        self._check(self._L.rwmi_set_concurrency(self._h, int(contexts)))
 
     def busy(self) -> bool:
         """True while GPU work of this context is in flight (rwmi_query, non-blocking)."""

@@ -35,12 +35,14 @@ class Backend:
     make(workload) -> sim. The sim has step(n) (asynchronous), busy() -> bool (non-blocking)
     and close(). footprint(workload) -> device bytes. chunk(workload) -> steps that one
     rwmi_step call must be a multiple of. collect(sim, workload) -> result dict, called once the
-    sim is idle after its last step.
+    sim is idle after its last step. share(sim, contexts), where given, is called before each
+    step with the number of contexts admitted then.
     """
     make: Callable
     footprint: Callable
     chunk: Callable
     collect: Callable
+    share: Optional[Callable] = None
 
 
 def gpu_backend(collect: Optional[Callable] = None) -> Backend:
@@ -63,7 +65,8 @@ def gpu_backend(collect: Optional[Callable] = None) -> Backend:
                 L = L * k // math.gcd(L, k)
         return L
 
-    return Backend(make, footprint, chunk, collect or default_collect)
+    return Backend(make, footprint, chunk, collect or default_collect,
+                   share=lambda sim, contexts: sim.set_concurrency(contexts))
 
 
 def default_collect(sim, w) -> dict:
@@ -257,6 +260,8 @@ class Server:
                         continue
                     if s.left > 0:
                         n = min(s.chunk, s.left)
+                        if be.share is not None:
+                            be.share(s.sim, len(active))
                         s.sim.step(n)
                         s.left -= n
                         still.append(s)
