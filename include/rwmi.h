@@ -317,7 +317,8 @@ RWMI_API rwmi_status rwmi_solid(rwmi_ctx* ctx, int32_t* count, int32_t* owner);
 
 /* IBB node classes of the current time (Section 2.4.3, the coupling = 1 reading): out[c] = 0 for a
  * fluid node, 1 + p when the cell centre lies inside particle p (Eq. 3 >= 1 in binary32, lowest
- * index). Computed on demand with any coupling. out: int32[ncell], host or device. */
+ * index). With that coupling they are the classes the last step (or the set-up) left for the next
+ * update; otherwise they are computed here. out: int32[ncell], host or device. */
 RWMI_API rwmi_status rwmi_nodes(rwmi_ctx* ctx, int32_t* out);
 
 /* {sum rho, sum_i f_i e_i (3 components)} over all cells at the last LBM step (FP64 sums;

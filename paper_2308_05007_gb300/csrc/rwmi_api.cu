@@ -1531,7 +1531,9 @@ RWMI_API rwmi_status rwmi_nodes(rwmi_ctx* c, int32_t* node) try {
   if (s != RWMI_OK) return s;
   uint16_t* tmp = (uint16_t*)c->scratch;
   if (c->P > 0) {
-    launch_nodes(c->g, particle_set(c), brick_set(c, par), tmp, c->stream);
+    // with the coupling, the classes the raster of this time wrote for the next step
+    if (c->cfg.coupling == 1) launch_read_nodes(c->g, brick_set(c, par), c->node[par], tmp, c->stream);
+    else launch_nodes(c->g, particle_set(c), brick_set(c, par), tmp, c->stream);
     c->launches++;
   } else {
     CK(cudaMemsetAsync(tmp, 0, sizeof(uint16_t) * n, c->stream));

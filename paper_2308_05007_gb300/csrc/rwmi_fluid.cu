@@ -911,8 +911,8 @@ void launch_density(int q, int storage, const Geom& g, const void* f, double rho
 
 // IBB node classes (Section 2.4.3) of every cell: a cell centre is solid when Eq. 3 of some particle
 // reaches 1 there (binary32, the CPU oracle's operation order), owned by the lowest such particle
-// index. Only cells of flagged bricks can be solid. Set-up and read-back; in a step the raster
-// writes the classes of flagged bricks and refill_kernel the rest. Brick-major: block 2 b + h takes
+// index. Only cells of flagged bricks can be solid. For the classes of t - 1 at set-up, and for
+// runs without the coupling; in a step the raster writes the classes of flagged bricks and refill_kernel the rest. Brick-major: block 2 b + h takes
 // half h (z rows 4 h .. 4 h + 3) of brick b.
 __global__ void __launch_bounds__(256) node_kernel(Geom g, ParticleSet ps, BrickSet bs, uint16_t* __restrict__ cur) {
   const uint32_t b = blockIdx.x >> 1;
@@ -940,6 +940,20 @@ __global__ void __launch_bounds__(256) node_kernel(Geom g, ParticleSet ps, Brick
     }
   }
   cur[c] = (uint16_t)node;
+}
+
+// The classes a step's raster left in nodes, with 0 in the bricks it did not write (read-back).
+__global__ void __launch_bounds__(256) read_nodes_kernel(Geom g, BrickSet bs, const uint16_t* __restrict__ nodes,
+                                                         uint16_t* __restrict__ out) {
+  const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= g.ncell) return;
+  const uint32_t z = fast_div(c, g.mxy, g.sxy), rem = c - z * g.nxy, y = fast_div(rem, g.mx, g.sx), x = rem - y * (uint32_t)g.n[0];
+  const bool held = bs.bword[((z >> 3) * (uint32_t)g.nb[1] + (y >> 3)) * (uint32_t)g.nb[0] + (x >> 3)] >> 16;
+  out[c] = held ? nodes[c] : (uint16_t)0;
+}
+
+void launch_read_nodes(const Geom& g, BrickSet bs, const uint16_t* nodes, uint16_t* out, cudaStream_t st) {
+  read_nodes_kernel<<<(g.ncell + 255) / 256, 256, 0, st>>>(g, bs, nodes, out);
 }
 
 void launch_nodes(const Geom& g, const ParticleSet& ps, BrickSet bs, uint16_t* cur, cudaStream_t st) {

@@ -355,8 +355,10 @@ void launch_dem_init(const DemArgs& a, cudaStream_t st);
 // body frames (cbody) and the state origins to the centres of mass
 void launch_dem_mass(const DemArgs& a, unsigned long long* sums, const double* density, double* mass, double* Ib,
                      double* props, float4* cbody, cudaStream_t st);
-// IBB node classes of all cells at the time of bricks bs into cur (set-up, read-back)
+// IBB node classes of all cells at the time of bricks bs into cur (set-up; read-back without the coupling)
 void launch_nodes(const Geom& g, const ParticleSet& ps, BrickSet bs, uint16_t* cur, cudaStream_t st);
+// The raster's classes of the time of bricks bs, completed with 0 in bricks without a particle, into out
+void launch_read_nodes(const Geom& g, BrickSet bs, const uint16_t* nodes, uint16_t* out, cudaStream_t st);
 // Completes the raster's classes cur of this time (0 in bricks without a particle); nodes solid in
 // prev and fluid now get the equilibrium at their former particle's rigid velocity (Eq. 27).
 void launch_refill(int q, int storage, const Geom& g, BrickSet bs, const uint16_t* prev, uint16_t* cur, void* f,
