@@ -575,9 +575,9 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     }
     // the partially saturated update through TMA-staged rows where it applies (same results).
     // Reduction steps run the update and the sums in one fused pass (binary32-shifted and
-    // binary64 storage): its update arithmetic is bit-identical to the plain update's, which a
-    // GPU test checks for every instantiation, so the trajectory does not depend on which steps
-    // are reduced; the other storages add the reduce-only pass.
+    // binary64 storage): its update stores the plain update's bits, which GPU tests check, so the
+    // trajectory does not depend on which steps are reduced (D3Q19 binary32 with IBB: but for
+    // binary32 rounding, about 1e-8 of a population); the other storages add the reduce-only pass.
     const bool staged = !ibb && !dem && c->tma_ok && c->cfg.lbm_staging;
     if (staged)
       launch_lbm_tma(c->cfg.q, c->cfg.storage, c->tmap[c->fcur], c->g, c->f[c->fcur], c->f[c->fcur ^ 1], c->u[tp],

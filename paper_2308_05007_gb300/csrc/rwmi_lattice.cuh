@@ -102,6 +102,13 @@ __device__ __forceinline__ void load_pose(const PoseF* pose, const PoseD* posed,
 }
 
 // Rigid velocity v_p + omega_p x (x - o_p) of particle p at the point (x, y, z), minimum image.
+// p + a b - c d; in binary64 with the two multiply-adds written out, so that every kernel that forms
+// a rigid velocity rounds it alike (the compiler may contract the plain form either way)
+template <typename R> __device__ __forceinline__ R cross_term(R p, R a, R b, R c, R d) {
+  if (sizeof(R) == 8) return fma(-c, d, fma(a, b, p));
+  return p + a * b - c * d;
+}
+
 template <typename R>
 __device__ __forceinline__ void rigid_velocity(const Geom& g, const PoseF* pose, const PoseD* posed, int p,
                                                R x, R y, R z, R* u) {
@@ -113,9 +120,9 @@ __device__ __forceinline__ void rigid_velocity(const Geom& g, const PoseF* pose,
       const R na = (R)g.n[a];
       if (r[a] > R(0.5) * na) r[a] -= na; else if (r[a] < -R(0.5) * na) r[a] += na;
     }
-  u[0] = pv[0] + pw[1] * r[2] - pw[2] * r[1];
-  u[1] = pv[1] + pw[2] * r[0] - pw[0] * r[2];
-  u[2] = pv[2] + pw[0] * r[1] - pw[1] * r[0];
+  u[0] = cross_term(pv[0], pw[1], r[2], pw[2], r[1]);
+  u[1] = cross_term(pv[1], pw[2], r[0], pw[0], r[2]);
+  u[2] = cross_term(pv[2], pw[0], r[1], pw[1], r[0]);
 }
 
 }  // namespace rwmi

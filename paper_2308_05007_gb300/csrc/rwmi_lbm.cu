@@ -362,8 +362,10 @@ __device__ __forceinline__ void lbm_body(Geom g, Planes<Q, typename Store<STORE>
   // cycles), so it works on the sums s_i = f_i + f_i' and differences d_i = f_i - f_i' of opposite
   // pairs: the moments need half the additions, and the even and odd parts of a pair's
   // post-collision values are formed once and added and subtracted. 96^3: 421 -> 305 us. Every
-  // multiply-add is written out, so that all instantiations round alike. (Binary32 keeps the
-  // direction-wise form and its rounding.)
+  // multiply-add of a stored value is written out, so that all instantiations store the same bits;
+  // forces may differ in their last bits. (Binary32 keeps the direction-wise form, which the
+  // compiler contracts; there the plain and the reducing update store the same bits but for D3Q19
+  // with IBB, whose populations differ by up to 1e-8.)
   constexpr bool PAIRS = sizeof(R) == 8;
   // moments (Eqs. 14-15); with shifted storage f holds f_i - w_i rho0
   R drho = R(0.0), jx = R(0.0), jy = R(0.0), jz = R(0.0);
@@ -440,9 +442,9 @@ __device__ __forceinline__ void lbm_body(Geom g, Planes<Q, typename Store<STORE>
             const R na = (R)g.n[a];
             if (r[a] > R(0.5) * na) r[a] -= na; else if (r[a] < -R(0.5) * na) r[a] += na;
           }
-        usx = pv[0] + pw[1] * r[2] - pw[2] * r[1];
-        usy = pv[1] + pw[2] * r[0] - pw[0] * r[2];
-        usz = pv[2] + pw[0] * r[1] - pw[1] * r[0];
+        usx = cross_term(pv[0], pw[1], r[2], pw[2], r[1]);
+        usy = cross_term(pv[1], pw[2], r[0], pw[0], r[2]);
+        usz = cross_term(pv[2], pw[0], r[1], pw[1], r[0]);
       }
     }
   }
@@ -456,13 +458,14 @@ __device__ __forceinline__ void lbm_body(Geom g, Planes<Q, typename Store<STORE>
   // velocity error against the FP64 oracle from 0.96e-5 to 1.5e-5 over 500 steps.
   // a solid node (IBB) holds the equilibrium at its particle's rigid velocity and rho0
   auto solid_eq = [&](R w, R eu, R uus) {
-    const R dev = R(3) * eu + R(4.5) * eu * eu - R(1.5) * uus;
+    const R dev = PAIRS ? fma(-R(1.5), uus, fma(R(3), eu, R(4.5) * eu * eu))
+                        : R(3) * eu + R(4.5) * eu * eu - R(1.5) * uus;
     return S::shifted ? w * rho0 * dev : w * rho0 * (R(1) + dev);
   };
   const R omB = R(1.0) - B;
   const R rtau = omB * omega;
   const R guo = omB * guo0;
-  const R om1 = R(1.0) - rtau;
+  const R om1 = PAIRS ? (R)__dsub_rn(1.0, (double)rtau) : R(1.0) - rtau;
   const R uF = PAIRS ? fma(uz, Fz, fma(uy, Fy, ux * Fx)) : ux * Fx + uy * Fy + uz * Fz;
   const R usus = PAIRS ? fma(usz, usz, fma(usy, usy, usx * usx)) : usx * usx + usy * usy + usz * usz;
   const R m15uu = -R(1.5) * uu;
@@ -571,7 +574,7 @@ __device__ __forceinline__ void lbm_body(Geom g, Planes<Q, typename Store<STORE>
       }
       if constexpr (decltype(sol)::value) {
         if (solid_self) {
-          const R eus = (R)ex * usx + (R)ey * usy + (R)ez * usz;
+          const R eus = PAIRS ? edot(ex, ey, ez, usx, usy, usz) : (R)ex * usx + (R)ey * usy + (R)ez * usz;
           out[i] = solid_eq(w, eus, usus);
           out[io] = solid_eq(w, -eus, usus);
         }
