@@ -98,7 +98,7 @@ def config_dict(a, w):
         "lbm_update": ("rows staged in shared memory by TMA tensor copies" if getattr(a, "lbm_staging", 0)
                        and w.storage in (0, 1, 2) and a.n % (8 if w.storage == 2 else 4) == 0
                        else "direct coalesced loads"),
-        "schedule": {0: "serial", 1: "raster of t+1 on a second stream beside the LBM of t",
+        "schedule": {0: "serial", 1: "raster of t+1 beside the LBM of t (programmatic launch)",
                      2: "raster of t+1 beside the LBM of t; walkers of t on their own stream beside "
                         "the fluid of t+1"}[getattr(a, "overlap", 2)],
     }

@@ -104,9 +104,10 @@ typedef struct {
                                   timing the update alone. */
     int32_t overlap;           /* step schedule, same results bit for bit in every case:
                                   0: one stream, phases one after the other;
-                                  1: the raster of t+1 on a second stream while the LBM of t runs
-                                     (ALU-bound beside HBM-bound);
-                                  2: as 1, and the walkers of t (with sort and moments) on a third
+                                  1: the raster of t+1 and, once its blocks are resident, the LBM of
+                                     t beside it (ALU-bound beside HBM-bound; with IBB or staging
+                                     the raster runs on a second stream instead);
+                                  2: as 1, and the walkers of t (with sort and moments) on their own
                                      stream beside the fluid of t+1. Default 2. */
     int32_t coupling;          /* particle-fluid coupling of the LBM: 0 partially saturated cells
                                   (Noble-Torczynski; default); 1 the paper's own (Section 2.4.3):

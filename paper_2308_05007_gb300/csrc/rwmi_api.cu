@@ -40,7 +40,10 @@ struct GraphKey {
   }
 };
 constexpr int64_t SEGMENT_MAX = 64;    // longest captured run of steps
-constexpr int PART_MIN = 8;             // SMs a context's raster and resolve grids are sized for at least
+// SMs a context's raster and resolve grids are sized for at least, however many step side by side. 64
+// domains of 16^3-48^3 as branches: 305 us per step with 19, 266 with 8, 262 with 3; a context left
+// alone in the end still has 16 raster blocks.
+constexpr int PART_MIN = 8;
 constexpr size_t GRAPH_CACHE_MAX = 32;  // captured runs kept per context; beyond, runs are eager
 
 struct GraphEntry {
@@ -63,7 +66,7 @@ struct rwmi_ctx {
                       // when many contexts step concurrently (rwmi_set_concurrency, branches of a batch)
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  cudaStream_t side = nullptr;    // raster of t+1 beside the LBM of t
+  cudaStream_t side = nullptr;    // raster of t+1 beside the LBM of t, with IBB or the staged update
   cudaStream_t wst = nullptr;     // walkers of t beside the fluid of t+1
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr, fluid_ev = nullptr, walk_ev[2] = {nullptr, nullptr};
   cudaEvent_t start_ev = nullptr;   // every block of the resolve pass has begun
@@ -610,16 +613,16 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     phase_end(c, RWMI_PHASE_RASTER);
   } else if (fork_raster && !ibb && !(c->tma_ok && c->cfg.lbm_staging)) {
     // the raster first, then the update as soon as the raster's blocks are resident: on two streams
-    // the update sometimes took every SM first, and the raster ran only as it drained (256^3: 707
-    // to 768 us per step from one build to the next; 708 us in this order, about 700 us with the
-    // present resolve pass). The walkers stay on their own stream: queued in this one, before the
-    // clear or behind the poses, runs at 256^3 took 2.5 to 7% longer.
+    // the update sometimes took every SM first, and the raster ran only as it drained (256^3: 707 to
+    // 768 us per step from one build to the next, 708 us in this order). The walkers stay on their
+    // own stream, where they fill what these leave free.
     pose();
-    // behind a pass 1 that filled every SM, the raster and the update wait until the resolve pass's
-    // blocks have begun: it is the chain the next step's walkers wait for, and on some GPUs the
-    // update's blocks took the SMs before it (256^3 run of 32 steps on such a GPU: 24.6 ms, 23.2 ms
-    // with the wait before the raster, 24.8 ms with it before the clear). A pass 1 that leaves
-    // SMs free leaves room for the resolve pass too, so small runs take no extra dependency.
+    // Behind a pass 1 that filled every SM, the raster and the update wait until the resolve pass's
+    // blocks have begun: it is the chain that the next step's walkers wait for. On most GPUs the wait
+    // changes nothing (256^3 with a quarter to eight times the walkers that fill the chip: within 0.5%
+    // always, never or by this rule); on some the update's blocks came first, for a reason not
+    // known, and 32 steps at 256^3 took 24.6 ms, 23.2 ms with the wait. A smaller pass 1 leaves SMs
+    // for the resolve pass, so small runs take no dependency they cannot need.
     if (c->start_rec) cudaStreamWaitEvent(c->stream, c->start_ev, 0);
     launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, part, c->stream);
     c->launches++;
@@ -1505,7 +1508,7 @@ RWMI_API rwmi_status rwmi_solid(rwmi_ctx* c, int32_t* count, int32_t* owner) try
   if (s != RWMI_OK) return s;
   int32_t* tmp = (int32_t*)c->scratch;   // the current time was rasterised by the last step / set-up
   if (c->cfg.coupling == 1 && c->P > 0) {
-    // IBB steps rasterise bricks and walker masks only: the counts of the current time are formed
+    // IBB steps write node classes and walker masks, not counts: the counts of the current time are formed
     // here, from its bricks (intact until the next step), by a full raster with a reset work
     // counter (it rewrites the same walker masks)
     CK(cudaMemsetAsync(c->bword[par] + c->nbrick + 1, 0, sizeof(uint32_t), c->stream));
@@ -2107,8 +2110,8 @@ RWMI_API rwmi_status rwmi_batch_step(rwmi_batch* b, int32_t nsteps) try {
       for (size_t k = 0; k < b->ctxs.size(); ++k) {
         rwmi_ctx* c = b->ctxs[k];
         cudaStreamWaitEvent(c->stream, b->fork, 0);
-        // Grids that fill the chip for one context only add work for many at a time (a raster cut into
-        // more pieces; 24 domains of 48^3-120^3: 1370 us per step, 1080 us with a part each).
+        // Grids that fill the chip for one context only add work for many at a time: a raster cut into
+        // more pieces (24 domains of 48^3-120^3: 1370 us per step, 1080 us with a part each).
         const int own = c->nsm_part;
         c->nsm_part = std::max(PART_MIN, c->nsm / (int)b->ctxs.size());
         for (int64_t st = 0; st < b->L; ++st) enqueue_step(c, st == b->L - 1);

@@ -644,10 +644,10 @@ int walker_grid(int64_t n, int nsm) {
   const int64_t blocks = (n + 255) / 256;
   return (int)(blocks < (int64_t)nsm * WALKER_BLOCKS_PER_SM ? blocks : (int64_t)nsm * WALKER_BLOCKS_PER_SM);
 }
-// The resolve pass runs beside the next step's fluid, so what it holds of an SM counts as much as
-// its own time: blocks of 128 threads at 48 registers, two waves of 10 per SM, measured best (256^3:
-// walker phase 251 us and step 704 us; 256 threads at 64 registers 257 / 773, 64 threads 255 / 706;
-// the loop-per-lane form at 32 registers 278 / 708; in a 33^3 box the walkers take 28 instead of 38 us)
+// The resolve pass runs beside the next step's fluid, so what it holds of an SM counts as much as its
+// own time: blocks of 128 threads at 48 registers, two waves of 10 per SM. At 256^3 the step takes
+// 704 us so, 706 with blocks of 64, 773 with 256 threads at 64 registers; its walkers 251 us alone (278
+// with a thread per walker that meets a particle).
 int resolve_grid(int nsm) { return nsm * 20; }
 
 bool walkers_fill_chip(int64_t n, int nsm) { return walker_grid(n, nsm) == nsm * WALKER_BLOCKS_PER_SM; }
