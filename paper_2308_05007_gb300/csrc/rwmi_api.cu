@@ -29,12 +29,13 @@ constexpr uint64_t CKPT_DEM_MAGIC = 0x314d4544ULL;  // "DEM1": the free-DEM sect
 // A captured run of steps is fixed by the buffer parities it starts from, its start time modulo
 // the chunk (which steps sort and form moments) and its length.
 struct GraphKey {
-  int fcur, pcur, part;
+  int fcur, pcur, part, waits;
   int64_t phase, len;
   bool operator<(const GraphKey& o) const {
     if (fcur != o.fcur) return fcur < o.fcur;
     if (pcur != o.pcur) return pcur < o.pcur;
     if (part != o.part) return part < o.part;
+    if (waits != o.waits) return waits < o.waits;
     if (phase != o.phase) return phase < o.phase;
     return len < o.len;
   }
@@ -132,6 +133,7 @@ struct rwmi_ctx {
   bool start_rec = false;              // start_ev likewise
   int fcur = 0, pcur = 0;
   int64_t binned_t = -1;
+  bool in_order = false;   // the walkers have been sorted by cell since they were set
   int64_t series_rows = 0;
   int64_t fseries_rows = 0;
   int64_t launches = 0;
@@ -479,6 +481,7 @@ rwmi_status alloc_walkers(rwmi_ctx* c, int64_t n) {
   c->nw = n;
   c->pcur = 0;
   c->binned_t = -1;
+  c->in_order = false;
   drop_graphs(c);
   // the flagged-walker list counters of both parities start at zero for new walkers
   CK(cudaMemsetAsync(c->wlist_n, 0, sizeof(unsigned int) * 2 * WLIST_STRIPES, c->stream));
@@ -494,6 +497,7 @@ void enqueue_sort(rwmi_ctx* c, cudaStream_t st) {
                  c->pos[c->pcur ^ 1], c->x0[c->pcur ^ 1], st);
   c->launches += 6;
   c->pcur ^= 1;
+  c->in_order = true;
 }
 
 void phase_begin(rwmi_ctx* c, int ph) {
@@ -510,6 +514,12 @@ bool force_recorded(const rwmi_ctx* c, int64_t done) {
 
 // Storages with the fused update-and-reduce pass (launch_lbm's `fused`).
 static bool fused_storage(int storage) { return storage == RWMI_STORE_FP32_SHIFT || storage == RWMI_STORE_FP64_SHIFT; }
+
+// Does the raster of the next step wait until the resolve pass of this one has begun? See enqueue_step.
+static bool raster_waits(const rwmi_ctx* c) {
+  return !c->timing && c->cfg.overlap >= 2 && c->P > 0 && c->cfg.coupling == 0 && !c->dem && c->in_order &&
+         walkers_fill_chip(c->nw, c->nsm);
+}
 
 // One timestep t -> t+1 of a run of steps (host mirrors advance as the launches are queued).
 // Buffers are per time parity where two steps' kernels may overlap: the solid fraction of t is
@@ -622,7 +632,9 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
     // changes nothing (256^3 with a quarter to eight times the walkers that fill the chip: within 0.5%
     // always, never or by this rule); on some the update's blocks came first, for a reason not
     // known, and 32 steps at 256^3 took 24.6 ms, 23.2 ms with the wait. A smaller pass 1 leaves SMs
-    // for the resolve pass, so small runs take no dependency they cannot need.
+    // for the resolve pass, so small runs take no dependency they cannot need. Nor do walkers that
+    // were never sorted: their scattered pass 1 takes four times as long, and the fluid that waits
+    // for it is not done beside it (the first 16 steps at 384^3: 105.9 ms with the wait, 90.9 without).
     if (c->start_rec) cudaStreamWaitEvent(c->stream, c->start_ev, 0);
     launch_raster(c->g, ps, brick_set(c, tn), c->solid[tn], c->status, part, c->stream);
     c->launches++;
@@ -653,7 +665,7 @@ void enqueue_step(rwmi_ctx* c, bool reduce) {
   }
   phase_begin(c, RWMI_PHASE_WALKERS);
   if (c->nw > 0) {
-    const bool ordered = ws != c->stream && fork_raster && !ibb && !dem && walkers_fill_chip(c->nw, c->nsm);
+    const bool ordered = raster_waits(c);
     launch_walkers(c->g, ps, brick_set(c, tn), c->pos[c->pcur], c->nw, c->u[tp], c->d_T, toff, tp, (float)c->D,
                    k0, k1, c->status, c->wlist, c->wlist_n, c->nsm, part, ws, ordered ? c->start_ev : nullptr);
     c->start_rec = ordered;
@@ -703,6 +715,7 @@ void advance_mirrors(rwmi_ctx* c, int64_t L) {
     c->t += 1;
     if (c->nw > 0 && c->cfg.sort_interval > 0 && c->t % c->cfg.sort_interval == 0) {
       c->pcur ^= 1;
+      c->in_order = true;
       c->binned_t = c->t;
     }
     if (c->cfg.moment_interval > 0 && c->t % c->cfg.moment_interval == 0) c->series_rows++;
@@ -1193,7 +1206,7 @@ RWMI_API rwmi_status rwmi_step(rwmi_ctx* c, int32_t n) try {
   while (n > 0) {
     const int64_t k = std::min<int64_t>(n, graphs ? G - c->t % L : n);
     n -= (int32_t)k;
-    const GraphKey key{c->fcur, c->pcur, c->nsm_part, c->t % L, k};
+    const GraphKey key{c->fcur, c->pcur, c->nsm_part, raster_waits(c) ? 1 : 0, c->t % L, k};
     auto it = graphs ? c->graphs.find(key) : c->graphs.end();
     if (graphs && it != c->graphs.end()) {
       CK(cudaGraphLaunch(it->second.exec, c->stream));
@@ -1728,6 +1741,7 @@ RWMI_API rwmi_status rwmi_load(rwmi_ctx* c, const char* path) try {
   c->fcur = (int)(c->t & 1);
   c->pcur = 0;
   c->binned_t = -1;
+  c->in_order = false;
   c->stepped = true;
   drop_graphs(c);
   CK(copy_now(c, c->f[c->fcur], f.data(), pop));
@@ -1936,6 +1950,7 @@ rwmi_status fused_capture(rwmi_batch* b, FusedGraph& fg) {
         scatter_args(rec(FP_SCATTER), c->g, c->pos[c->pcur], c->x0[c->pcur], c->nw, c->offsets, c->rank,
                      c->pos[c->pcur ^ 1], c->x0[c->pcur ^ 1]);
         c->pcur ^= 1;
+        c->in_order = true;
         c->binned_t = c->t;
       }
       const bool mom = c->cfg.moment_interval > 0 && c->t % c->cfg.moment_interval == 0;
@@ -2100,7 +2115,12 @@ RWMI_API rwmi_status rwmi_batch_step(rwmi_batch* b, int32_t nsteps) try {
   }
   for (int32_t done_steps = 0; done_steps < nsteps; done_steps += (int32_t)b->L) {
     std::vector<int> key;
-    for (rwmi_ctx* c : b->ctxs) { key.push_back(c->fcur); key.push_back(c->pcur); c->stepped = true; }
+    for (rwmi_ctx* c : b->ctxs) {
+      key.push_back(c->fcur);
+      key.push_back(c->pcur);
+      key.push_back(raster_waits(c) ? 1 : 0);
+      c->stepped = true;
+    }
     auto it = b->graphs.find(key);
     if (it == b->graphs.end()) {
       std::vector<int64_t> l0;
