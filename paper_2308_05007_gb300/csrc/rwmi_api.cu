@@ -41,10 +41,11 @@ struct GraphKey {
   }
 };
 constexpr int64_t SEGMENT_MAX = 64;    // longest captured run of steps
-// SMs a context's raster and resolve grids are sized for at least, however many step side by side. 64
-// domains of 16^3-48^3 as branches: 305 us per step with 19, 266 with 8, 262 with 3; a context left
-// alone in the end still has 16 raster blocks.
-constexpr int PART_MIN = 8;
+// SMs a context's raster and resolve grids are sized for at least, however many step side by side
+// (8 raster blocks, 80 of the resolve pass). As branches of a batch, ms per step for 64 domains of
+// 48^3-160^3 / 256 of 16^3-48^3 / 64 of 16^3-48^3: 3.98 / 1.12 / 0.278 with 2, 4.03 / 1.11 / 0.252 with
+// 4, 4.15 / 1.21 / 0.267 with 8; the served stream takes the same with 2 to 8.
+constexpr int PART_MIN = 4;
 constexpr size_t GRAPH_CACHE_MAX = 32;  // captured runs kept per context; beyond, runs are eager
 
 struct GraphEntry {
