@@ -467,8 +467,8 @@ struct RasterWarp {
 // work (up to ~100 evaluations of 64 sub-samples, ~1 us each), so a list shorter than four per
 // resident warp is spread over them: slices of 32, 16 or 8 mini-bricks, then parts that share out a
 // slice's straddling mini-bricks down to one each. Every piece stages the candidates again, so
-// longer lists keep whole bricks (256^3, 13175 bricks on 2432 warps: 190 us whole, 267 us in
-// eighths; 96^3, 902 bricks: 97 us whole, 43 us in eighths).
+// longer lists keep whole bricks (256^3, 13175 bricks on 2432 warps: 183 us whole, 241 us in
+// eighths; 96^3, 902 bricks: 75 us whole, 40 us in eighths).
 __device__ __forceinline__ int raster_pieces_log2(uint32_t nlist, uint32_t warps) {
   int s = 0;
   while (s < 6 && (nlist << (s + 1)) <= 4u * warps) ++s;
